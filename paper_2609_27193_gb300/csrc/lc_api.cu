@@ -777,7 +777,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         d.numel = s.numel;
         d.lead = int32_t((uintptr_t(s.w) & 15) >> esz_log2);
         d.esz_log2 = esz_log2;
-        d.coaligned = s.snap && (uintptr_t(s.w) & 15) == (uintptr_t(s.snap) & 15);
+        d.rshift = s.snap ? int32_t((uintptr_t(s.snap) - uintptr_t(s.w)) & 15) : 0;
         d.layer = s.layer;
         d.nvec = (int64_t(d.lead) + s.numel + ve - 1) / ve;
         d.vec_begin = V;

@@ -34,7 +34,8 @@ struct SegDev {
     int64_t nvec;        // number of vectors covering the segment
     int32_t lead;        // elements of vector 0 in front of the segment start
     int32_t esz_log2;    // 1 = bf16, 2 = fp32
-    int32_t coaligned;   // w and r have the same address modulo 16
+    int32_t rshift;      // (address of r - address of w) mod 16: R's bytes for vector k start this
+                         // many bytes into a 16-byte window (0: w and r are co-aligned)
     int32_t layer;
 };
 

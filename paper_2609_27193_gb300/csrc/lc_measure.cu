@@ -19,6 +19,8 @@
 #include "lc_bulk.cuh"
 #include "lc_reduce.cuh"
 
+#include <type_traits>
+
 namespace lc {
 namespace {
 
@@ -138,7 +140,7 @@ __device__ void process_run(const SegDev& sd, int64_t lo, int64_t hi, double& dd
     const int ve = 16 >> sd.esz_log2;
     const bool head_partial = sd.lead > 0;
     const bool tail_partial = ((int64_t(sd.lead) + sd.numel) % ve) != 0;
-    if (sd.coaligned) {
+    if (sd.rshift == 0) {
         const int64_t kf0 = head_partial ? 1 : 0;
         const int64_t kf1 = tail_partial ? sd.nvec - 1 : sd.nvec;
         const int64_t a = lo > kf0 ? lo : kf0;
@@ -199,13 +201,27 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // then units of a pool of small ranges, each taken from a counter
 // (next_pool_range), so that CTAs streaming faster take more of the work.
 // Each range is the same walk over segment runs as above, turned into a
-// sequence of jobs by one producer thread (warp 0): for the full co-aligned
-// vectors of a run, chunks of up to
+// sequence of jobs by one producer thread (warp 0): for the vectors of a run
+// that lie inside W and whose R windows (below) lie inside R, chunks of up to
 // kMChunk bytes of W and the same bytes of R loaded by cp.async.bulk into a
 // ring of kMStages buffers (one "full" mbarrier per buffer, completed by the
-// loads' byte count); for partial edge vectors and runs whose W and R are
-// not co-aligned, a job the consumers read from global memory element by
-// element; after each run a flush.  Warps 1..7 consume every job in order:
+// loads' byte count); for the few vectors at a segment's edges, a job the
+// consumers read from global memory element by element; after each run a
+// flush.
+//
+// W and R at different offsets from a 16-byte boundary (rshift != 0: weights
+// that are views of a flat buffer, snapshots that are tensors of their own):
+// a bulk load starts on 16 bytes, so R's chunk is loaded from the boundary
+// below its first byte, one vector longer, and the consumers take R's vector
+// v from the staged vectors v and v + 1, shifted by rshift bytes.  The shift
+// is the same for the whole segment, so it is a template parameter of the
+// loop.  A run like that used to be read element by element, two fp64 adds
+// each: a decision over 412 M bf16 parameters in 146 such segments took
+// 3110 us and takes 315 us (0.53 and 5.2 TB/s; the same parameters co-aligned
+// 265).  What bounds the shifted runs is the consumers' arithmetic: with plain
+// fp32 chains, as in the aligned runs, it took 277 us, but then lost precision
+// against the element path's fp64 (6e-12 instead of 3e-12 off the exact sums),
+// so the chains keep their rounding errors.  Warps 1..7 consume every job in order:
 // each thread adds its 16-byte vectors of the chunk into fp32 lanes (at most
 // ceil(chunk vectors / 224) terms before they go to fp64), and at a flush
 // each warp reduces its threads' fp64 sums in a fixed order into the run
@@ -227,7 +243,8 @@ constexpr int kMStages = LC_MEASURE_BULK_STAGES;
 constexpr uint32_t kMChunk = LC_MEASURE_BULK_CHUNK;      // bytes of W (and of R) per buffer
 constexpr int kMConsumerWarps = kMeasureThreads / 32 - 1;   // warps 1.. consume (2.. in accumulate mode)
 constexpr int kMConsumers = 32 * kMConsumerWarps;
-constexpr size_t kMeasureBulkSmem = size_t(kMStages) * 2 * kMChunk;
+constexpr uint32_t kMStage = 2 * kMChunk + 128;          // R's part has room for the window's extra vector
+constexpr size_t kMeasureBulkSmem = size_t(kMStages) * kMStage;
 static_assert(kMChunk % 16 == 0 && kMStages >= 2, "measure ring shape");
 
 enum : int32_t { kJobChunk = 0, kJobScalar = 1, kJobFlush = 2, kJobEnd = 3 };
@@ -238,6 +255,8 @@ struct MJob {
     int32_t seg;
     int32_t slot;       // first partial slot of the run (flush)
     int32_t esz_log2;   // element size of the segment (chunk)
+    int32_t rshift;     // the segment's rshift (chunk)
+    int32_t pad;
 };
 
 struct MRing {
@@ -260,12 +279,13 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
         r.jobs[st] = j;
         if (j.kind == kJobChunk) {
             const uint32_t bytes = uint32_t(j.k1 - j.k0) * 16u;
+            const uint32_t rbytes = bytes + (sd.rshift ? 16u : 0u);
             const uint8_t* wb = sd.w - (int64_t(sd.lead) << sd.esz_log2) + 16 * j.k0;
-            const uint8_t* rb = sd.r - (int64_t(sd.lead) << sd.esz_log2) + 16 * j.k0;
-            mbar_expect_tx(full_s + 8 * st, 2 * bytes + (stall ? 16u : 0u));
+            const uint8_t* rb = sd.r - (int64_t(sd.lead) << sd.esz_log2) - sd.rshift + 16 * j.k0;
+            mbar_expect_tx(full_s + 8 * st, bytes + rbytes + (stall ? 16u : 0u));
             stall = false;
-            bulk_g2s(ring_s + uint32_t(st) * 2 * kMChunk, wb, bytes, full_s + 8 * st);
-            bulk_g2s(ring_s + uint32_t(st) * 2 * kMChunk + kMChunk, rb, bytes, full_s + 8 * st);
+            bulk_g2s(ring_s + uint32_t(st) * kMStage, wb, bytes, full_s + 8 * st);
+            bulk_g2s(ring_s + uint32_t(st) * kMStage + kMChunk, rb, rbytes, full_s + 8 * st);
         } else {
             mbar_arrive(full_s + 8 * st);
         }
@@ -285,37 +305,199 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
             const int64_t seg_end = sd.vec_begin + sd.nvec;
             const int64_t lo = v0 - sd.vec_begin;
             const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
-            const int ve = 16 >> sd.esz_log2;
-            const bool head_partial = sd.lead > 0;
-            const bool tail_partial = ((int64_t(sd.lead) + sd.numel) % ve) != 0;
-            if (sd.coaligned) {
-                if (head_partial && lo <= 0 && 0 < hi) ok = post({0, 1, kJobScalar, s, slot, 0}, sd);
-                const int64_t kf0 = head_partial ? 1 : 0;
-                const int64_t kf1 = tail_partial ? sd.nvec - 1 : sd.nvec;
-                const int64_t a = lo > kf0 ? lo : kf0;
-                const int64_t e = hi < kf1 ? hi : kf1;
-                constexpr int64_t kCV = kMChunk / 16;
-                for (int64_t x = a; ok && x < e; x += kCV)
-                    ok = post({x, (x + kCV < e ? x + kCV : e), kJobChunk, s, slot, sd.esz_log2}, sd);
-                const int64_t last = sd.nvec - 1;
-                if (ok && tail_partial && last >= lo && last < hi && !(head_partial && last == 0))
-                    ok = post({last, last + 1, kJobScalar, s, slot, 0}, sd);
-            } else {
-                ok = post({lo, hi, kJobScalar, s, slot, 0}, sd);
-            }
-            if (ok) ok = post({0, 0, kJobFlush, s, slot, 0}, sd);
+            // vectors [kf0, kf1) lie inside W with their R windows inside R
+            const int64_t lead_b = (int64_t(sd.lead) << sd.esz_log2) + sd.rshift;
+            const int64_t kf0 = (lead_b + 15) >> 4;
+            int64_t kf1 = ((lead_b + (sd.numel << sd.esz_log2)) >> 4) - (sd.rshift ? 1 : 0);
+            if (kf1 < kf0) kf1 = kf0;
+            const int64_t a = lo > kf0 ? lo : kf0;
+            const int64_t e = hi < kf1 ? hi : kf1;
+            if (lo < kf0) ok = post({lo, (hi < kf0 ? hi : kf0), kJobScalar, s, slot, 0, 0, 0}, sd);
+            constexpr int64_t kCV = kMChunk / 16;
+            for (int64_t x = a; ok && x < e; x += kCV)
+                ok = post({x, (x + kCV < e ? x + kCV : e), kJobChunk, s, slot, sd.esz_log2, sd.rshift, 0}, sd);
+            if (ok && hi > kf1) ok = post({(lo > kf1 ? lo : kf1), hi, kJobScalar, s, slot, 0, 0, 0}, sd);
+            if (ok) ok = post({0, 0, kJobFlush, s, slot, 0, 0, 0}, sd);
             slot += kMeasureBulkSlotsPerRun;
             ++s;
             v0 = sd.vec_begin + hi;
         }
     }
-    if (ok) ok = post({0, 0, kJobEnd, 0, 0, 0}, sd);
+    if (ok) ok = post({0, 0, kJobEnd, 0, 0, 0, 0, 0}, sd);
     if (!ok) {
         raise_fault(p.fault);
         // the loads of the last kMStages jobs may still be landing in shared memory
         const uint64_t first = k > uint64_t(kMStages) ? k - kMStages : 0;
         for (uint64_t c = first; c < k; ++c)
             mbar_wait_bounded(full_s + 8 * int(c % kMStages), uint32_t((c / kMStages) & 1), kDrainNs);
+    }
+}
+
+// Bytes [SH, SH + 16) of the 32 bytes of a and b (SH even).
+template <int SH>
+__device__ __forceinline__ uint4 window16(const uint4& a, const uint4& b) {
+    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    constexpr int q = SH / 4;
+    if constexpr (SH % 4 == 0) {
+        return make_uint4(x[q], x[q + 1], x[q + 2], x[q + 3]);
+    } else {
+        return make_uint4(__funnelshift_r(x[q], x[q + 1], 16), __funnelshift_r(x[q + 1], x[q + 2], 16),
+                          __funnelshift_r(x[q + 2], x[q + 3], 16), __funnelshift_r(x[q + 3], x[q + 4], 16));
+    }
+}
+
+// a + b, its rounding error added to e (exact in any order of magnitude).
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = a + b, t = s - a;
+    e += (a - (s - t)) + (b - t);
+    return s;
+}
+
+// The same in three operations: exact once the sum a is at least as large as
+// the term b; before that within half the error that plain addition makes.
+__device__ __forceinline__ float fast_two_sum(float a, float b, float& e) {
+    const float s = a + b;
+    e += b - (s - a);
+    return s;
+}
+
+// One chunk's fp32 chains of a thread with their rounding errors.  bf16
+// terms have 8 significant bits, so a chain rounds only where two terms are
+// more than 2^16 apart and the short form serves; fp32 terms round in every
+// addition and there are half as many of them per byte.
+template <int ESZ_LOG2>
+struct CompSums {
+    static constexpr int kLanes = 16 >> ESZ_LOG2;
+    float s[kLanes], e[kLanes];
+    __device__ __forceinline__ CompSums() {
+#pragma unroll
+        for (int i = 0; i < kLanes; ++i) { s[i] = 0.f; e[i] = 0.f; }
+    }
+    __device__ __forceinline__ void add(int i, float x) {
+        s[i] = ESZ_LOG2 == 1 ? fast_two_sum(s[i], x, e[i]) : two_sum(s[i], x, e[i]);
+    }
+    // the chains' sum, left in s[0] and e[0]
+    __device__ __forceinline__ void reduce() {
+#pragma unroll
+        for (int k = kLanes / 2; k > 0; k >>= 1) {
+#pragma unroll
+            for (int i = 0; i < k; ++i) {
+                e[i] += e[i + k];
+                s[i] = two_sum(s[i], s[i + k], e[i]);
+            }
+        }
+    }
+};
+
+template <int ESZ_LOG2>
+__device__ __forceinline__ void accumulate_comp(const uint4& w, const uint4& r, CompSums<ESZ_LOG2>& cd,
+                                                CompSums<ESZ_LOG2>& ca) {
+    const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
+    const uint32_t rv[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if constexpr (ESZ_LOG2 == 1) {
+            const float r0 = bf16_lo(rv[j]), r1 = bf16_hi(rv[j]);
+            cd.add(2 * j, fabsf(bf16_lo(wv[j]) - r0));
+            cd.add(2 * j + 1, fabsf(bf16_hi(wv[j]) - r1));
+            ca.add(2 * j, fabsf(r0));
+            ca.add(2 * j + 1, fabsf(r1));
+        } else {
+            const float r0 = __uint_as_float(rv[j]);
+            cd.add(j, fabsf(__uint_as_float(wv[j]) - r0));
+            ca.add(j, fabsf(r0));
+        }
+    }
+}
+
+// The same vectors element by element in fp64, for a chain that is not
+// finite: terms near the end of fp32's range, an infinity or a NaN.
+template <int ESZ_LOG2>
+__device__ __noinline__ double2 staged_elements(const uint8_t* W, const uint8_t* R, int n, int tid, int nt) {
+    double dd = 0.0, da = 0.0;
+    for (int v = tid; v < n; v += nt) {
+        for (int i = 0; i < (16 >> ESZ_LOG2); ++i) {
+            const int64_t e = int64_t(v) * (16 >> ESZ_LOG2) + i;
+            const float w = load_elem(W, ESZ_LOG2, e), r = load_elem(R, ESZ_LOG2, e);
+            dd += double(fabsf(w - r));
+            da += double(fabsf(r));
+        }
+    }
+    return make_double2(dd, da);
+}
+
+// n staged vectors of a run whose R bytes start SH bytes into their windows.
+// In accumulate mode R's 16-byte vector v of the chunk (at r_out + 16 v)
+// takes the end of W's vector v - 1 and the start of vector v; the chunk's
+// first and last R vectors are only partly its own and are stored by
+// elements.  No other chunk reads or writes those elements of R.
+//
+// The fp32 chains keep their rounding errors (comp_add): these runs used to
+// be added element by element in fp64, and the sums are no less exact now.
+template <int ESZ_LOG2, int SH, bool WRITE_R, int NT>
+__device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int n, int tid, uint8_t* r_out,
+                                            double& dd, double& da, float& ed, float& ea) {
+    CompSums<ESZ_LOG2> cd, ca;
+#pragma unroll 2
+    for (int v = tid; v < n; v += NT) {
+        const uint4 w = W[v];
+        accumulate_comp<ESZ_LOG2>(w, window16<SH>(R[v], R[v + 1]), cd, ca);
+        if constexpr (WRITE_R) {
+            using T = typename std::conditional<ESZ_LOG2 == 1, uint16_t, uint32_t>::type;
+            constexpr int kE = 16 >> ESZ_LOG2, kSplit = kE - (SH >> ESZ_LOG2);
+            const uint32_t x[4] = {w.x, w.y, w.z, w.w};
+            auto elem = [&](int i) {
+                return T(ESZ_LOG2 == 1 ? x[i >> 1] >> (16 * (i & 1)) : x[ESZ_LOG2 == 1 ? 0 : i]);
+            };
+            if (v > 0) {
+                st_vec(r_out + 16 * v, window16<16 - SH>(W[v - 1], w));
+            } else {
+                T* first = reinterpret_cast<T*>(r_out + SH);
+#pragma unroll
+                for (int i = 0; i < kSplit; ++i) first[i] = elem(i);
+            }
+            if (v == n - 1) {
+                T* last = reinterpret_cast<T*>(r_out + 16 * n);
+#pragma unroll
+                for (int i = kSplit; i < kE; ++i) last[i - kSplit] = elem(i);
+            }
+        }
+    }
+    cd.reduce();
+    ca.reduce();
+    if (isfinite(cd.s[0]) && isfinite(ca.s[0])) {
+        dd += double(cd.s[0]);
+        da += double(ca.s[0]);
+        ed += cd.e[0];
+        ea += ca.e[0];
+    } else {
+        const double2 x = staged_elements<ESZ_LOG2>(reinterpret_cast<const uint8_t*>(W),
+                                                    reinterpret_cast<const uint8_t*>(R) + SH, n, tid, NT);
+        dd += x.x;
+        da += x.y;
+    }
+}
+
+template <bool WRITE_R, int NT>
+__device__ __forceinline__ void shifted_chunk(int esz_log2, int rshift, const uint4* W, const uint4* R, int n,
+                                              int tid, uint8_t* r_out, double& dd, double& da,
+                                              float& ed, float& ea) {
+    if (esz_log2 == 1) {
+        switch (rshift) {
+            case 2: shifted_run<1, 2, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 4: shifted_run<1, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 6: shifted_run<1, 6, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 8: shifted_run<1, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 10: shifted_run<1, 10, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 12: shifted_run<1, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            default: shifted_run<1, 14, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+        }
+    } else {
+        switch (rshift) {
+            case 4: shifted_run<2, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 8: shifted_run<2, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            default: shifted_run<2, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+        }
     }
 }
 
@@ -328,6 +510,7 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
     const int tid = int(threadIdx.x) - 32 * kFirstWarp;
     const int warp = tid >> 5, lane = tid & 31;
     double dd = 0.0, da = 0.0;
+    float ed = 0.f, ea = 0.f;   // rounding errors of the run's compensated chains
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kMStages);
         const uint32_t parity = uint32_t((k / kMStages) & 1);
@@ -342,25 +525,38 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
         const MJob j = r.jobs[st];
         if (j.kind == kJobEnd) break;
         if (j.kind == kJobChunk) {
-            const uint4* W = reinterpret_cast<const uint4*>(ring + size_t(st) * 2 * kMChunk);
+            const uint4* W = reinterpret_cast<const uint4*>(ring + size_t(st) * kMStage);
             const uint4* R = W + kMChunk / 16;
             const int n = int(j.k1 - j.k0);
-            float ad[8], aa[8];
-#pragma unroll
-            for (int q = 0; q < 8; ++q) { ad[q] = 0.f; aa[q] = 0.f; }
-            if (j.esz_log2 == 1) {
-#pragma unroll 4
-                for (int v = tid; v < n; v += kThreads) accumulate<1>(W[v], R[v], ad, aa);
+            if (j.rshift) {
+                uint8_t* r_out = nullptr;
+                if constexpr (WRITE_R) {
+                    const SegDev& sd = p.segs[j.seg];
+                    r_out = sd.r - (int64_t(sd.lead) << sd.esz_log2) - sd.rshift + 16 * j.k0;
+                }
+                shifted_chunk<WRITE_R, kThreads>(j.esz_log2, j.rshift, W, R, n, tid, r_out, dd, da, ed, ea);
             } else {
+                float ad[8], aa[8];
+#pragma unroll
+                for (int q = 0; q < 8; ++q) { ad[q] = 0.f; aa[q] = 0.f; }
+                if (j.esz_log2 == 1) {
 #pragma unroll 4
-                for (int v = tid; v < n; v += kThreads) accumulate<2>(W[v], R[v], ad, aa);
+                    for (int v = tid; v < n; v += kThreads) accumulate<1>(W[v], R[v], ad, aa);
+                } else {
+#pragma unroll 4
+                    for (int v = tid; v < n; v += kThreads) accumulate<2>(W[v], R[v], ad, aa);
+                }
+                dd += double(tree8(ad));
+                da += double(tree8(aa));
             }
-            dd += double(tree8(ad));
-            da += double(tree8(aa));
         } else if (j.kind == kJobScalar) {
             const SegDev sd = p.segs[j.seg];
             for (int64_t v = j.k0 + tid; v < j.k1; v += kThreads) scalar_vector<WRITE_R>(sd, v, dd, da);
         } else {   // flush: this warp's share of the run, in a fixed order
+            dd += double(ed);
+            da += double(ea);
+            ed = 0.f;
+            ea = 0.f;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
                 dd += __shfl_down_sync(0xffffffffu, dd, off);
@@ -391,12 +587,12 @@ __device__ void measure_store_r(const MeasureParams& p, const uint8_t* ring, MRi
         }
         const MJob j = r.jobs[st];
         if (j.kind == kJobEnd) break;
-        if (j.kind == kJobChunk) {
+        if (j.kind == kJobChunk && j.rshift == 0) {
             const SegDev sd = p.segs[j.seg];
             uint8_t* rb = sd.r - (int64_t(sd.lead) << sd.esz_log2) + 16 * j.k0;
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(rb),
-                         "r"(ring_s + uint32_t(st) * 2 * kMChunk), "r"(uint32_t(j.k1 - j.k0) * 16u)
+                         "r"(ring_s + uint32_t(st) * kMStage), "r"(uint32_t(j.k1 - j.k0) * 16u)
                          : "memory");
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");

@@ -240,7 +240,7 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         d.numel = s.numel;
         d.lead = int32_t((reinterpret_cast<uintptr_t>(s.w) & 15) >> esz_log2);
         d.esz_log2 = esz_log2;
-        d.coaligned = (reinterpret_cast<uintptr_t>(s.w) & 15) == (reinterpret_cast<uintptr_t>(s.snap) & 15);
+        d.rshift = int32_t((reinterpret_cast<uintptr_t>(s.snap) - reinterpret_cast<uintptr_t>(s.w)) & 15);
         d.layer = s.layer;
         d.nvec = (int64_t(d.lead) + s.numel + ve - 1) / ve;
     }
