@@ -370,6 +370,7 @@ struct lc_ctx {
     int measure_grid = 0, copy_grid = 0, nslots = 0;
     int bulk_grid = 0;                     // CTAs of a bulk-engine copy launch
     bool bulk_sources = false;             // every registered array is device memory
+    bool off16 = false;                    // some registered array starts off a 16-byte boundary
     uint32_t* h_fault = nullptr;           // pinned, mapped: a bulk copy gave up waiting
     uint32_t* d_fault = nullptr;           // its device address
     uint32_t* d_fault_dev = nullptr;       // its copy in device memory (read by every copy CTA)
@@ -472,7 +473,7 @@ cudaError_t launch_copy_engine(lc_ctx* ctx, CopyParams p, bool bulk, uint64_t un
     ctx->counters.kernel_launches += 1;
     ctx->counters.copy_launches += 1;
     if (bulk) ctx->counters.bulk_copy_launches += 1;
-    return bulk ? launch_copy_bulk(p, grid, s) : launch_copy(p, grid, s);
+    return bulk ? launch_copy_bulk(p, grid, ctx->off16, s) : launch_copy(p, grid, s);
 }
 
 // Copy trace.  A span's start event is recorded on its stream right before
@@ -760,6 +761,14 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     ctx->order = order;
     ctx->snap_missing = false;
     for (int32_t i = 0; i < nseg; ++i) ctx->snap_missing |= segs[i].snap == nullptr;
+    // Bulk stores need 16-byte addresses: with one array off them the copies
+    // take the kernel that shifts.  The line lies at one array because that
+    // kernel loses next to nothing on aligned entries: a 1.2 G parameter step
+    // with a quarter of the layers packed takes 2362 us with it, 2355 without.
+    ctx->off16 = false;
+    for (int32_t i = 0; i < nseg; ++i)
+        ctx->off16 |= ((uintptr_t(segs[i].w) | uintptr_t(segs[i].snap) | uintptr_t(segs[i].exp_avg) |
+                        uintptr_t(segs[i].exp_avg_sq)) & 15) != 0;
     ctx->layer_seg_begin.assign(nlayers + 1, 0);
     for (int32_t i = 0; i < nseg; ++i) ctx->layer_seg_begin[ctx->segs[i].layer + 1] += 1;
     for (int32_t l = 0; l < nlayers; ++l) ctx->layer_seg_begin[l + 1] += ctx->layer_seg_begin[l];

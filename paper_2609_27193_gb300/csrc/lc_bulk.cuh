@@ -1,7 +1,8 @@
 // lc_bulk.cuh -- the bulk-copy engine pieces shared by the kernels that
 // stream global memory through shared-memory rings (lc_copy.cu: the pack,
 // commit and restore; lc_measure.cu: the Eq. 1 scan): mbarrier waits that
-// give up after a bound, cp.async.bulk loads and stores, and the fault word.
+// give up after a bound, cp.async.bulk loads and stores, the fault word, and
+// 16-byte windows at any even offset in staged bytes.
 #pragma once
 
 #include "lc_internal.cuh"
@@ -71,6 +72,19 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src, uin
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst_smem),
         "l"(src), "r"(bytes), "r"(bar)
         : "memory");
+}
+
+// Bytes [SH, SH + 16) of the 32 bytes of a and b (SH even).
+template <int SH>
+__device__ __forceinline__ uint4 window16(const uint4& a, const uint4& b) {
+    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    constexpr int q = SH / 4;
+    if constexpr (SH % 4 == 0) {
+        return make_uint4(x[q], x[q + 1], x[q + 2], x[q + 3]);
+    } else {
+        return make_uint4(__funnelshift_r(x[q], x[q + 1], 16), __funnelshift_r(x[q + 1], x[q + 2], 16),
+                          __funnelshift_r(x[q + 2], x[q + 3], 16), __funnelshift_r(x[q + 3], x[q + 4], 16));
+    }
 }
 
 // Records that a bounded wait ran out: the host reads the word (host-mapped).

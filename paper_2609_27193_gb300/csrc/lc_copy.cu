@@ -2,7 +2,8 @@
 // state into one contiguous stream), the snapshot commit and the restore
 // scatter (§3.5): copy_bulk_kernel (the payload goes through shared memory
 // on the bulk-copy engine; the default whenever every address is device
-// memory) and copy_kernel (every thread loads and stores 16-byte vectors;
+// memory), copy_shift_kernel (its form for layouts with arrays off 16-byte
+// boundaries: bulk loads, vector stores) and copy_kernel (every thread loads and stores 16-byte vectors;
 // used for host memory and on request).
 //
 // A launch covers the work range [lo, hi) of a descriptor list whose
@@ -441,6 +442,226 @@ __global__ void __launch_bounds__(kCopyThreads, 1) copy_bulk_kernel(CopyParams p
     walk_entries<kWorkers, true>(p, first, x, xe, int(threadIdx.x) - 64);
 }
 
+// ---------------------------------------------------------------------------
+// Copies of arrays that do not start on 16-byte boundaries (tensors that are
+// views of a flat buffer, shards of a tensor).  The bulk engine moves whole
+// 16-byte granules, so only the load side uses it here: the granules of the
+// source that lie inside the entry stream through the same ring, and the
+// consumer warps (2..7) write them to each destination in vectors aligned
+// there, a vector taken from two staged ones at the offset between source and
+// destination (one switch per chunk, since the offset is the same for the
+// whole entry).  The bytes before the first and after the last granule, and
+// the padding of GATHER, are warp 1's.  Such entries used to move in units of
+// 2 or 4 bytes with ordinary loads: packing a quarter of the layers of a
+// 412 M parameter shard took 1960 us and takes 550 (the whole step 2256 and
+// 848 us; the same tensors on 16-byte boundaries 841).  Like the bulk form it
+// is bound by DRAM.
+// ---------------------------------------------------------------------------
+constexpr int kShiftFirstWarp = 2;
+constexpr int kShiftWarps = BS / 32 - kShiftFirstWarp;
+constexpr int kShiftThreads = 32 * kShiftWarps;
+
+struct ShiftJob {
+    uint8_t* dst;       // where the first staged byte goes
+    uint8_t* dst2;      // or null
+    uint32_t bytes;     // staged bytes, a multiple of 16; 0: end of the range
+};
+
+struct ShiftRing {
+    uint64_t full[kStages];
+    uint64_t empty[kStages];
+    ShiftJob jobs[kStages];
+};
+
+// The payload [lo, hi) of an entry that the launch covers, and [g0, g1), the
+// whole granules of its source (g1 <= g0: none).
+struct Staged {
+    int64_t lo, hi, g0, g1;
+};
+__device__ __forceinline__ Staged staged_range(const CopyParams& p, const CopyDesc& d, const uint8_t* src) {
+    Staged t;
+    t.lo = d.woff < p.lo ? int64_t(p.lo - d.woff) : 0;
+    t.hi = int64_t(p.hi - d.woff < d.nbytes ? p.hi - d.woff : d.nbytes);
+    t.g0 = t.lo + int64_t((16 - (uintptr_t(src) & 15)) & 15);
+    t.g1 = t.hi - int64_t((uintptr_t(src) + uint64_t(t.hi)) & 15);
+    return t;
+}
+
+// A CTA's share [a, b) of an entry (multiples of 16, as is lo) stands for the
+// staged bytes [a, b) + (g0 - lo), cut off at g1.  The bytes before g0 belong
+// to the CTA whose share starts at lo, those from g1 on to the one whose
+// share holds the last byte.
+struct ShiftCursor {
+    int i;
+    uint64_t x;
+    int64_t cur, end;      // staged bytes still to load of the entry before i
+    EntryAddr e;
+};
+
+__device__ bool shift_next(const CopyParams& p, ShiftCursor& c, uint64_t xe, ShiftJob& j, const uint8_t*& src) {
+    while (c.cur >= c.end) {
+        if (c.x >= xe || c.i >= p.ndesc) return false;
+        const CopyDesc d = p.desc[c.i++];
+        const uint64_t ent_end = d.woff + d.span;
+        if (ent_end <= c.x) continue;
+        const uint64_t end = xe < ent_end ? xe : ent_end;
+        c.e = entry_addr(p, d);
+        const Staged t = staged_range(p, d, c.e.src);
+        c.cur = int64_t(c.x - d.woff) + (t.g0 - t.lo);
+        c.end = int64_t(end - d.woff) + (t.g0 - t.lo);
+        if (c.end > t.g1) c.end = t.g1;
+        c.x = end;
+    }
+    const int64_t n = c.end - c.cur < int64_t(kChunk) ? c.end - c.cur : int64_t(kChunk);
+    src = c.e.src + c.cur;
+    j.dst = c.e.dst + c.cur;
+    j.dst2 = c.e.dst2 ? c.e.dst2 + c.cur : nullptr;
+    j.bytes = uint32_t(n);
+    c.cur += n;
+    return true;
+}
+
+__device__ void shift_produce(const CopyParams& p, int i, uint64_t x, uint64_t xe, uint32_t ring_s, ShiftRing& r) {
+    const uint32_t full_s = smem_addr(r.full), empty_s = smem_addr(r.empty);
+    ShiftCursor c;
+    c.i = i;
+    c.x = x;
+    c.cur = c.end = 0;
+    ShiftJob j;
+    const uint8_t* src = nullptr;
+    bool have = shift_next(p, c, xe, j, src);
+    for (uint64_t k = 0;; ++k) {
+        const int s = int(k % kStages);
+        if (k >= uint64_t(kStages) &&
+            !mbar_wait_bounded(empty_s + 8 * s, uint32_t((k / kStages - 1) & 1), kWaitNs)) {
+            raise_copy_fault(p);
+            // the loads of the last kStages chunks may still be landing in shared memory
+            const uint64_t first = k > uint64_t(kStages) ? k - kStages : 0;
+            for (uint64_t q = first; q < k; ++q)
+                mbar_wait_bounded(full_s + 8 * int(q % kStages), uint32_t((q / kStages) & 1), kDrainNs);
+            return;
+        }
+        if (!have) {
+            r.jobs[s].bytes = 0;
+            mbar_arrive(full_s + 8 * s);
+            return;
+        }
+        r.jobs[s] = j;
+        mbar_expect_tx(full_s + 8 * s, j.bytes + (p.stall_first && k == 0 ? 16u : 0u));
+        bulk_g2s(ring_s + uint32_t(s) * kChunk, src, j.bytes, full_s + 8 * s);
+        have = shift_next(p, c, xe, j, src);
+    }
+}
+
+// n staged bytes to dst, SH bytes short of a 16-byte boundary.
+template <int SH>
+__device__ __forceinline__ void put_shifted(const uint8_t* staged, uint32_t n, uint8_t* dst, int tid) {
+    const uint4* S = reinterpret_cast<const uint4*>(staged);
+    const int nv = int(n / 16) - (SH ? 1 : 0);
+#pragma unroll 4
+    for (int v = tid; v < nv; v += kShiftThreads) {
+        if constexpr (SH == 0) st_v4(dst + 16 * v, S[v]);
+        else st_v4(dst + SH + 16 * v, window16<SH>(S[v], S[v + 1]));
+    }
+    if constexpr (SH != 0) {
+        // the vectors that this chunk shares with its neighbours, in 2-byte units
+        const int u = tid < SH / 2 ? tid : tid < 8 ? int(n / 2) - 8 + tid : -1;
+        if (u >= 0) reinterpret_cast<uint16_t*>(dst)[u] = reinterpret_cast<const uint16_t*>(staged)[u];
+    }
+}
+
+__device__ __forceinline__ void put_staged(const uint8_t* staged, uint32_t n, uint8_t* dst, int tid) {
+    switch ((16 - (uintptr_t(dst) & 15)) & 15) {
+        case 0: put_shifted<0>(staged, n, dst, tid); break;
+        case 2: put_shifted<2>(staged, n, dst, tid); break;
+        case 4: put_shifted<4>(staged, n, dst, tid); break;
+        case 6: put_shifted<6>(staged, n, dst, tid); break;
+        case 8: put_shifted<8>(staged, n, dst, tid); break;
+        case 10: put_shifted<10>(staged, n, dst, tid); break;
+        case 12: put_shifted<12>(staged, n, dst, tid); break;
+        default: put_shifted<14>(staged, n, dst, tid); break;
+    }
+}
+
+__device__ void shift_consume(const CopyParams& p, const uint8_t* ring, ShiftRing& r) {
+    const uint32_t full_s = smem_addr(r.full), empty_s = smem_addr(r.empty);
+    const int tid = int(threadIdx.x) - 32 * kShiftFirstWarp, lane = tid & 31;
+    for (uint64_t k = 0;; ++k) {
+        const int s = int(k % kStages);
+        const uint32_t parity = uint32_t((k / kStages) & 1);
+        int ok = 1;
+        if (lane == 0) ok = mbar_wait_bounded(full_s + 8 * s, parity, kWaitNs) ? 1 : 0;
+        ok = __shfl_sync(0xffffffffu, ok, 0);
+        if (!ok) {
+            if (lane == 0) raise_copy_fault(p);
+            break;
+        }
+        mbar_try_wait(full_s + 8 * s, parity);   // completed: orders this lane's reads after the loads
+        const ShiftJob j = r.jobs[s];
+        if (j.bytes == 0) break;
+        const uint8_t* staged = ring + size_t(s) * kChunk;
+        put_staged(staged, j.bytes, j.dst, tid);
+        if (j.dst2) put_staged(staged, j.bytes, j.dst2, tid);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty_s + 8 * s);
+    }
+}
+
+// Warp 1: payload bytes [u, v) of an entry in 2-byte units (every address of
+// an entry is a multiple of its element size), and the padding.
+__device__ __forceinline__ void edge_units(const EntryAddr& e, int64_t u, int64_t v, int lane) {
+    for (int64_t q = u + 2 * lane; q < v; q += 64) {
+        const uint16_t x = *reinterpret_cast<const uint16_t*>(e.src + q);
+        *reinterpret_cast<uint16_t*>(e.dst + q) = x;
+        if (e.dst2) *reinterpret_cast<uint16_t*>(e.dst2 + q) = x;
+    }
+}
+
+__device__ void shift_edges(const CopyParams& p, int i, uint64_t x, uint64_t xe, int lane) {
+    for (; x < xe && i < p.ndesc; ++i) {
+        const CopyDesc d = p.desc[i];
+        const uint64_t ent_end = d.woff + d.span;
+        if (ent_end <= x) continue;
+        const uint64_t end = xe < ent_end ? xe : ent_end;
+        const int64_t a = int64_t(x - d.woff), b = int64_t(end - d.woff), nb = int64_t(d.nbytes);
+        const EntryAddr e = entry_addr(p, d);
+        const Staged t = staged_range(p, d, e.src);
+        const bool last = a < t.hi && t.hi <= b;
+        if (t.g1 <= t.g0) {
+            if (last) edge_units(e, t.lo, t.hi, lane);
+        } else {
+            if (a == t.lo) edge_units(e, t.lo, t.g0, lane);
+            if (last) edge_units(e, t.g1, t.hi, lane);
+        }
+        if (p.mode == kGather && b > nb)
+            for (int64_t q = (a > nb ? a : nb) + 2 * lane; q < b; q += 64)
+                *reinterpret_cast<uint16_t*>(e.dst + q) = 0;
+        x = end;
+    }
+}
+
+__global__ void __launch_bounds__(kCopyThreads, 1) copy_shift_kernel(CopyParams p) {
+    extern __shared__ __align__(128) uint8_t ring[];
+    __shared__ __align__(8) ShiftRing r;
+    __shared__ uint32_t s_abort;
+    uint64_t x, xe;
+    int first;
+    if (!cta_range(p, x, xe, first)) return;
+    if (threadIdx.x == 0) {
+        s_abort = p.fault_dev ? *reinterpret_cast<volatile const uint32_t*>(p.fault_dev) : 0u;
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(smem_addr(&r.full[s]), 1);
+            mbar_init(smem_addr(&r.empty[s]), kShiftWarps);
+        }
+        mbar_init_fence();
+    }
+    __syncthreads();
+    if (s_abort) return;
+    if (threadIdx.x == 0) shift_produce(p, first, x, xe, smem_addr(ring), r);
+    else if (threadIdx.x >= 32 * kShiftFirstWarp) shift_consume(p, ring, r);
+    else if (threadIdx.x >= 32) shift_edges(p, first, x, xe, int(threadIdx.x) - 32);
+}
+
 }  // namespace
 
 cudaError_t launch_copy(const CopyParams& p, int grid, cudaStream_t s) {
@@ -453,15 +674,18 @@ cudaError_t copy_occupancy(int* blocks_per_sm) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, copy_kernel, kCopyThreads, 0);
 }
 
-cudaError_t launch_copy_bulk(const CopyParams& p, int grid, cudaStream_t s) {
+cudaError_t launch_copy_bulk(const CopyParams& p, int grid, bool shifted, cudaStream_t s) {
     cudaGetLastError();
-    copy_bulk_kernel<<<grid, kCopyThreads, kBulkSmem, s>>>(p);
+    if (shifted) copy_shift_kernel<<<grid, kCopyThreads, kBulkSmem, s>>>(p);
+    else copy_bulk_kernel<<<grid, kCopyThreads, kBulkSmem, s>>>(p);
     return cudaGetLastError();
 }
 
 cudaError_t copy_bulk_prepare(int* blocks_per_sm) {
     cudaError_t e = cudaFuncSetAttribute(copy_bulk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          int(kBulkSmem));
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(copy_shift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBulkSmem));
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, copy_bulk_kernel, kCopyThreads,
                                                          kBulkSmem);

@@ -224,7 +224,8 @@ cudaError_t copy_occupancy(int* blocks_per_sm);
 // Bulk-engine copy (cp.async.bulk through shared memory); every address the
 // launch touches must be device memory.  copy_bulk_prepare raises the
 // kernel's shared-memory limit and reports its CTAs per SM.
-cudaError_t launch_copy_bulk(const CopyParams& p, int grid, cudaStream_t s);
+// `shifted`: the form for layouts with arrays off 16-byte boundaries.
+cudaError_t launch_copy_bulk(const CopyParams& p, int grid, bool shifted, cudaStream_t s);
 cudaError_t copy_bulk_prepare(int* blocks_per_sm);
 
 // Sets the thread-local message returned by lc_last_error().

@@ -218,7 +218,7 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // loop.  A run like that used to be read element by element, two fp64 adds
 // each: a decision over 412 M bf16 parameters in 146 such segments took
 // 3110 us and takes 315 us (0.53 and 5.2 TB/s; the same parameters co-aligned
-// 265).  What bounds the shifted runs is the consumers' arithmetic: with plain
+// 277).  What bounds the shifted runs is the consumers' arithmetic: with plain
 // fp32 chains, as in the aligned runs, it took 277 us, but then lost precision
 // against the element path's fp64 (6e-12 instead of 3e-12 off the exact sums),
 // so the chains keep their rounding errors.  Warps 1..7 consume every job in order:
@@ -330,19 +330,6 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
         const uint64_t first = k > uint64_t(kMStages) ? k - kMStages : 0;
         for (uint64_t c = first; c < k; ++c)
             mbar_wait_bounded(full_s + 8 * int(c % kMStages), uint32_t((c / kMStages) & 1), kDrainNs);
-    }
-}
-
-// Bytes [SH, SH + 16) of the 32 bytes of a and b (SH even).
-template <int SH>
-__device__ __forceinline__ uint4 window16(const uint4& a, const uint4& b) {
-    const uint32_t x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-    constexpr int q = SH / 4;
-    if constexpr (SH % 4 == 0) {
-        return make_uint4(x[q], x[q + 1], x[q + 2], x[q + 3]);
-    } else {
-        return make_uint4(__funnelshift_r(x[q], x[q + 1], 16), __funnelshift_r(x[q + 1], x[q + 2], 16),
-                          __funnelshift_r(x[q + 2], x[q + 3], 16), __funnelshift_r(x[q + 3], x[q + 4], 16));
     }
 }
 

@@ -101,3 +101,76 @@ def test_measure_of_extreme_values_off_alignment(what, value):
     assert np.array_equal(got[0], [want, 0.0, n], equal_nan=True)
     assert got[1].tolist() == [n * 0.25, n * 0.25, n]
     lc.close()
+
+
+@pytest.mark.parametrize("staging", [0, 2 << 20])
+@pytest.mark.parametrize("fuse", [True, False])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_pack_commit_restore_off_alignment(dtype, fuse, staging):
+    """Weights, references and moments each at their own offset from a
+    16-byte boundary: the packed stream (to the device, or through a store
+    with `staging` bytes of ring, whose launches end inside sections), the
+    committed references and the restored tensors equal the sources byte for
+    byte, padding is zero and nothing beside them is written."""
+    torch = require_gpu()
+    import paper_2609_27193_gb300 as P
+    esz = 2 if dtype == "bf16" else 4
+    tt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(esz + fuse)
+    sizes = [1, 2, 7, 8, 9, 17, 33, 63, 64, 65, 24575, 24576, 24577, 1000003]
+    segs, keep = [], []
+    for k, n in enumerate(sizes * (16 // esz // 2)):
+        offs = (esz * k % 16, esz * (k // 2 + k // len(sizes)) % 16, 4 * k % 16, 4 * (k + k // 3) % 16)
+        part = [_placed(torch, n, d, o) + (o,) for d, o in zip((tt, tt, torch.float32, torch.float32), offs)]
+        for _, view, _ in part:
+            view.copy_(torch.randn(n, generator=g, device="cuda"))
+        keep.append(part)
+        segs.append(P.segment(k // 3, part[0][1], part[1][1], part[2][1], part[3][1]))
+    N = segs[-1].layer + 1
+    more = dict(staging_bytes=staging) if staging else {}
+    lc = P.LayerCheck(fuse_commit=fuse, **more)
+    lc.register_layout(segs, N)
+    lc.measure(1)
+    mask, _, nbytes = lc.select(1e-3, 0)
+    assert mask.all()
+    raw = lambda x: x.contiguous().view(torch.uint8)
+    want = []
+    for l in range(N):
+        members = [keep[k] for k, s in enumerate(segs) if s.layer == l]
+        for part in (0, 2, 3):
+            for m in members:
+                b = raw(m[part][1])
+                want.append(b)
+                want.append(torch.zeros(-b.numel() % 256, dtype=torch.uint8, device="cuda"))
+    want = torch.cat(want)
+    assert want.numel() == nbytes
+    src = [[p[1].clone() for p in part] for part in keep]
+    if staging:
+        store = P.Store(lc, capacity_bytes=nbytes + (1 << 20))
+        lc.pack_async(store)
+    else:
+        dst = torch.full((nbytes + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        lc.pack_device(dst)
+    lc.commit_snapshot()
+    if staging:
+        lc.wait_durable(1)
+        got = np.concatenate([store.block(i) for i in range(len(store))])
+        assert np.array_equal(got, want.cpu().numpy())
+    else:
+        torch.cuda.synchronize()
+        assert torch.equal(dst[:nbytes], want) and set(dst[nbytes:].tolist()) == {0xA5}
+    for part, old in zip(keep, src):
+        assert torch.equal(raw(part[1][1]), raw(old[0])), "reference"
+        if staging:
+            for x in part:
+                x[1].zero_()
+    if staging:
+        torch.cuda.synchronize()
+        lc.restore(store, 1)
+        for part, old in zip(keep, src):
+            for j, k in ((0, 0), (1, 0), (2, 2), (3, 3)):
+                assert torch.equal(raw(part[j][1]), raw(old[k])), "restored"
+    for part in keep:
+        for buf, view, o in part:
+            assert set(_outside(buf, view, o)) == {0xA5}, "bytes beside a tensor were written"
+    lc.close()
