@@ -219,12 +219,14 @@ __global__ void __launch_bounds__(kMeasureThreads, LC_ADAM_MIN_BLOCKS) adamw_mea
 // in flight (registers bound it).  Here one producer thread (warp 0) streams
 // chunks of kAChunkVec vectors of w, m, v and the gradient into a ring of
 // kAStages shared-memory buffers with cp.async.bulk, so the bytes in flight
-// no longer cost registers; seven consumer warps take each chunk from
-// shared memory, run the same element step, store w, m, v and the bf16
-// model copy with ordinary 16- and 8-byte stores, and add the Eq. 1 sums of
-// the update.  Edge vectors, segments whose arrays do not line up and
-// gradient vectors that would start a bulk copy off a 16-byte boundary go
-// element by element.  Partition (with its pool of units), jobs, the run
+// no longer cost registers; six consumer warps (2..7) take each chunk from
+// shared memory, run the same element step, put the updated w, m and v back
+// into the buffer, store the bf16 model copy themselves and add the Eq. 1
+// sums of the update; warp 1 writes the buffer's w, m and v with bulk stores.
+// A bulk copy starts on 16 bytes: an array that does not line up with w's
+// vectors is loaded from the granule below its chunk (Window).  Vectors at a
+// segment's edges whose windows would leave an array go element by element.
+// Partition (with its pool of units), jobs, the run
 // box that combines the warps' partial sums, and bounded waits are those of
 // the bulk-load measure.
 // ---------------------------------------------------------------------------
@@ -234,73 +236,115 @@ __global__ void __launch_bounds__(kMeasureThreads, LC_ADAM_MIN_BLOCKS) adamw_mea
 #ifndef LC_ADAM_BULK_VECS
 #define LC_ADAM_BULK_VECS 512
 #endif
-// 1: the updated w, m and v go back into the buffer and one thread (warp 1)
-// writes them with bulk stores; 0: the consumers store them themselves.
-#ifndef LC_ADAM_BULK_STORE
-#define LC_ADAM_BULK_STORE 1
-#endif
-constexpr bool kABulkStore = LC_ADAM_BULK_STORE != 0;
 constexpr int kAStages = LC_ADAM_BULK_STAGES;
 constexpr int kAChunkVec = LC_ADAM_BULK_VECS;                 // vectors of 4 parameters per chunk
-constexpr uint32_t kAStage = uint32_t(kAChunkVec) * 64u;      // w, m, v and gradient, 16 B each per vector
+constexpr uint32_t kAPart = 16u * uint32_t(kAChunkVec) + 16u;   // an array's chunk, and a window's extra vector
+constexpr uint32_t kAStage = 4u * kAPart;                     // w, m, v and gradient
 constexpr size_t kAdamBulkSmem = size_t(kAStages) * kAStage;
-constexpr int kAFirstConsumerWarp = kABulkStore ? 2 : 1;
+constexpr int kAFirstConsumerWarp = 2;     // warp 0 loads, warp 1 stores
 constexpr int kAConsumerWarps = kMeasureThreads / 32 - kAFirstConsumerWarp;
 constexpr int kAConsumers = 32 * kAConsumerWarps;
 static_assert(kAChunkVec % 2 == 0 && kAStages >= 2, "fused ring shape");
 
 enum : int32_t { kAJobChunk = 0, kAJobScalar = 1, kAJobFlush = 2, kAJobEnd = 3 };
+// Which arrays line up with w's vectors: m, v, gradient and model copy; m and v; not even those.
+enum : int32_t { kALined = 0, kAMoments = 1, kALoose = 2 };
 
+// What the producer knows of a job travels with it: the consumers and the
+// storer read no table in global memory per chunk.
 struct AJob {
-    int64_t k0, k1;
+    int64_t k0, k1;      // element-wise job: vectors [k0, k1) of the segment
+    uint8_t *w, *m, *v;  // chunk: where its vectors go
+    uint8_t* model;      // or null
     int32_t kind;
     int32_t seg;
     int32_t slot;
+    int32_t n;           // chunk: vectors
+    int32_t form;        // chunk: kALined, kAMoments or kALoose
+    int32_t grad_bf16;
+    int32_t grad_off;    // chunk: place of its first gradient in the first staged granule
     int32_t pad;
 };
 
 struct ARing {
     uint64_t full[kAStages];
-    uint64_t computed[kAStages];   // consumers done with the buffer (bulk-store form)
+    uint64_t computed[kAStages];   // consumers done with the buffer
     uint64_t empty[kAStages];
     AJob jobs[kAStages];
     RunBox<kAStages, kAConsumerWarps> box;
 };
+
+// Vectors [k0, k0 + n) of an array of `per_vec` bytes a vector whose first
+// element belongs to vector 0 at place `lead`: the 16-byte granules that hold
+// them, and how far into the first one they start.
+struct Window {
+    const uint8_t* from;
+    uint32_t off, bytes;
+    __device__ __forceinline__ Window(const uint8_t* base, int64_t lead, int per_vec, int64_t k0, uint32_t n) {
+        const uint8_t* first = base - lead * (per_vec / 4) + per_vec * k0;
+        off = uint32_t(uintptr_t(first) & 15);
+        from = first - off;
+        bytes = (off + uint32_t(per_vec) * n + 15u) & ~15u;
+    }
+};
+
+// Narrows [kf0, kf1) to the vectors whose windows lie inside the array.
+__device__ __forceinline__ void window_bounds(const void* array, const SegDev& sd, int per_vec, int64_t& kf0,
+                                              int64_t& kf1) {
+    const int64_t at = int64_t(uintptr_t(array) & 15);                  // addresses relative to the granule below
+    const int64_t zero = at - int64_t(sd.lead) * (per_vec / 4);         // of vector 0
+    const int64_t lo = ((at + 15) & ~int64_t(15)) - zero + per_vec - 1;
+    const int64_t hi = ((at + sd.numel * (per_vec / 4)) & ~int64_t(15)) - zero;
+    if (lo / per_vec > kf0) kf0 = lo / per_vec;
+    if (hi / per_vec < kf1) kf1 = hi / per_vec;
+}
 
 __device__ void adam_produce(const MeasureParams& p, const OptSegDev* opt, uint8_t* ring, ARing& r) {
     const uint32_t ring_s = smem_addr(ring);
     const uint32_t full_s = smem_addr(r.full), empty_s = smem_addr(r.empty);
     uint64_t k = 0;
     bool stall = p.stall_first != 0;
-    auto post = [&](const AJob& j, const SegDev& sd, const OptSegDev& od) -> bool {
+    SegDev sd{};
+    OptSegDev od{};
+    auto post = [&](int32_t kind, int32_t s, int32_t slot, int64_t k0, int64_t k1) -> bool {
         const int st = int(k % kAStages);
         if (k >= uint64_t(kAStages) &&
             !mbar_wait_bounded(empty_s + 8 * st, uint32_t((k / kAStages - 1) & 1), kWaitNs))
             return false;
-        r.jobs[st] = j;
-        if (j.kind == kAJobChunk) {
-            const uint32_t n = uint32_t(j.k1 - j.k0);
+        AJob& j = r.jobs[st];
+        j.kind = kind;
+        j.seg = s;
+        j.slot = slot;
+        if (kind == kAJobChunk) {
+            const uint32_t n = uint32_t(k1 - k0);
             const int64_t lead = sd.lead;
-            const uint32_t gsz = od.grad_bf16 ? 8u : 16u;
             const uint32_t buf = ring_s + uint32_t(st) * kAStage;
-            mbar_expect_tx(full_s + 8 * st, n * (48u + gsz) + (stall ? 16u : 0u));
+            const Window wm(reinterpret_cast<const uint8_t*>(od.m), lead, 16, k0, n);
+            const Window wv(reinterpret_cast<const uint8_t*>(od.v), lead, 16, k0, n);
+            const Window wg(od.grad, lead, od.grad_bf16 ? 8 : 16, k0, n);
+            j.w = const_cast<uint8_t*>(sd.w) - 4 * lead + 16 * k0;
+            j.m = const_cast<uint8_t*>(wm.from) + wm.off;
+            j.v = const_cast<uint8_t*>(wv.from) + wv.off;
+            j.model = od.model ? od.model - 2 * lead + 8 * k0 : nullptr;
+            j.n = int32_t(n);
+            j.form = od.fast ? kALined : (wm.off | wv.off) == 0 ? kAMoments : kALoose;
+            j.grad_bf16 = od.grad_bf16;
+            j.grad_off = int32_t(wg.off);
+            mbar_expect_tx(full_s + 8 * st, 16 * n + wm.bytes + wv.bytes + wg.bytes + (stall ? 16u : 0u));
             stall = false;
-            bulk_g2s(buf, sd.w - 4 * lead + 16 * j.k0, 16 * n, full_s + 8 * st);
-            bulk_g2s(buf + 16 * kAChunkVec, reinterpret_cast<const uint8_t*>(od.m) - 4 * lead + 16 * j.k0,
-                     16 * n, full_s + 8 * st);
-            bulk_g2s(buf + 32 * kAChunkVec, reinterpret_cast<const uint8_t*>(od.v) - 4 * lead + 16 * j.k0,
-                     16 * n, full_s + 8 * st);
-            bulk_g2s(buf + 48 * kAChunkVec, od.grad - (od.grad_bf16 ? 2 : 4) * lead + int64_t(gsz) * j.k0,
-                     gsz * n, full_s + 8 * st);
+            bulk_g2s(buf, j.w, 16 * n, full_s + 8 * st);
+            bulk_g2s(buf + kAPart, wm.from, wm.bytes, full_s + 8 * st);
+            bulk_g2s(buf + 2 * kAPart, wv.from, wv.bytes, full_s + 8 * st);
+            bulk_g2s(buf + 3 * kAPart, wg.from, wg.bytes, full_s + 8 * st);
         } else {
+            j.k0 = k0;
+            j.k1 = k1;
             mbar_arrive(full_s + 8 * st);
         }
         ++k;
         return true;
     };
     bool ok = true;
-    SegDev sd{};
-    OptSegDev od{};
     // the CTA's own range, then units of the pool until it is empty
     for (int rng = int(blockIdx.x); ok && rng >= 0; rng = ok ? next_pool_range(p) : -1) {
         int64_t v0 = p.cta_vec_begin[rng];
@@ -313,49 +357,162 @@ __device__ void adam_produce(const MeasureParams& p, const OptSegDev* opt, uint8
             const int64_t seg_end = sd.vec_begin + sd.nvec;
             const int64_t lo = v0 - sd.vec_begin;
             const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
-            const bool head_partial = sd.lead > 0;
-            const bool tail_partial = ((int64_t(sd.lead) + sd.numel) % 4) != 0;
-            if (od.fast) {
-                if (head_partial && lo <= 0 && 0 < hi) ok = post({0, 1, kAJobScalar, s, slot, 0}, sd, od);
-                const int64_t kf0 = head_partial ? 1 : 0;
-                const int64_t kf1 = tail_partial ? sd.nvec - 1 : sd.nvec;
-                int64_t x = lo > kf0 ? lo : kf0;
-                const int64_t e = hi < kf1 ? hi : kf1;
-                // a bf16 gradient vector is 8 bytes: a bulk copy must start on 16
-                const uintptr_t gb = uintptr_t(od.grad) - 2 * uintptr_t(sd.lead);
-                if (ok && od.grad_bf16 && x < e && ((gb + 8 * uintptr_t(x)) & 15)) {
-                    ok = post({x, x + 1, kAJobScalar, s, slot, 0}, sd, od);
-                    ++x;
-                }
-                while (ok && x < e) {
-                    int64_t n = e - x < kAChunkVec ? e - x : kAChunkVec;
-                    if (od.grad_bf16 && (n & 1)) n -= 1;      // the gradient bytes stay a multiple of 16
-                    if (n == 0) {
-                        ok = post({x, x + 1, kAJobScalar, s, slot, 0}, sd, od);
-                        ++x;
-                        continue;
-                    }
-                    ok = post({x, x + n, kAJobChunk, s, slot, 0}, sd, od);
-                    x += n;
-                }
-                const int64_t last = sd.nvec - 1;
-                if (ok && tail_partial && last >= lo && last < hi && !(head_partial && last == 0))
-                    ok = post({last, last + 1, kAJobScalar, s, slot, 0}, sd, od);
-            } else {
-                ok = post({lo, hi, kAJobScalar, s, slot, 0}, sd, od);
-            }
-            if (ok) ok = post({0, 0, kAJobFlush, s, slot, 0}, sd, od);
+            // vectors [kf0, kf1) lie inside w with their windows inside m, v and the gradient
+            int64_t kf0 = sd.lead > 0 ? 1 : 0;
+            int64_t kf1 = (int64_t(sd.lead) + sd.numel) / 4;
+            window_bounds(od.m, sd, 16, kf0, kf1);
+            window_bounds(od.v, sd, 16, kf0, kf1);
+            window_bounds(od.grad, sd, od.grad_bf16 ? 8 : 16, kf0, kf1);
+            if (kf1 < kf0) kf1 = kf0;
+            if (lo < kf0) ok = post(kAJobScalar, s, slot, lo, (hi < kf0 ? hi : kf0));
+            const int64_t e = hi < kf1 ? hi : kf1;
+            for (int64_t x = lo > kf0 ? lo : kf0; ok && x < e; x += kAChunkVec)
+                ok = post(kAJobChunk, s, slot, x, (x + kAChunkVec < e ? x + kAChunkVec : e));
+            if (ok && hi > kf1) ok = post(kAJobScalar, s, slot, (lo > kf1 ? lo : kf1), hi);
+            if (ok) ok = post(kAJobFlush, s, slot, 0, 0);
             slot += kMeasureBulkSlotsPerRun;
             ++s;
             v0 = sd.vec_begin + hi;
         }
     }
-    if (ok) ok = post({0, 0, kAJobEnd, 0, 0, 0}, sd, od);
+    if (ok) ok = post(kAJobEnd, 0, 0, 0, 0);
     if (!ok) {
         raise_fault(p.fault);
         const uint64_t first = k > uint64_t(kAStages) ? k - kAStages : 0;
         for (uint64_t c = first; c < k; ++c)
             mbar_wait_bounded(full_s + 8 * int(c % kAStages), uint32_t((c / kAStages) & 1), kDrainNs);
+    }
+}
+
+__device__ __forceinline__ uint4 words4(const uint32_t* w) { return make_uint4(w[0], w[1], w[2], w[3]); }
+
+// The updated vector q of m or v (first staged word at w, which is `off`
+// bytes into its granule): the words stay where they were read, for the
+// storer; those outside the chunk's whole granules go to global memory here.
+__device__ __forceinline__ void put_words(uint32_t* w, uint8_t* global, uint32_t off, int q, int n,
+                                          const float (&x)[4]) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        w[e] = __float_as_uint(x[e]);
+        if (off && ((q == 0 && off + 4 * e < 16) || (q == n - 1 && off + 4 * e >= 16)))
+            *reinterpret_cast<float*>(global + 16 * int64_t(q) + 4 * e) = x[e];
+    }
+}
+
+// The model copy's four bf16 at any 2-byte boundary.
+__device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi) {
+    if ((uintptr_t(to) & 7) == 0) {
+        st_u2(to, make_uint2(lo, hi));
+    } else if ((uintptr_t(to) & 3) == 0) {
+        reinterpret_cast<uint32_t*>(to)[0] = lo;
+        reinterpret_cast<uint32_t*>(to)[1] = hi;
+    } else {
+        *reinterpret_cast<uint16_t*>(to) = uint16_t(lo);
+        *reinterpret_cast<uint32_t*>(to + 2) = (lo >> 16) | (hi << 16);
+        *reinterpret_cast<uint16_t*>(to + 6) = uint16_t(hi >> 16);
+    }
+}
+
+// One staged chunk.  In kALined, m, v, the gradient and the model copy
+// line up with w's vectors.  Otherwise the gradient (and in kALoose m and v)
+// starts where it likes: its staged words are read, and m's and v's written
+// back, one by one (stride-4 words: four-way bank conflicts), and the Eq. 1 chains keep their rounding errors -- such segments used to be added
+// element by element in fp64, and the sums are no less exact now.  %FIGURE%
+template <int FORM>
+__device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid, const AdamConsts& c, double& dd,
+                                           double& da, float& ed, float& ea) {
+    constexpr bool LINED = FORM == kALined, MOMENTS = FORM != kALoose;
+    const int n = j.n;
+    uint4* W = reinterpret_cast<uint4*>(buf);
+    const uint32_t om = MOMENTS ? 0u : uint32_t(uintptr_t(j.m) & 15), ov = MOMENTS ? 0u : uint32_t(uintptr_t(j.v) & 15);
+    const uint32_t og = uint32_t(j.grad_off);
+    uint8_t* Mb = buf + kAPart + om;
+    uint8_t* Vb = buf + 2 * kAPart + ov;
+    const uint8_t* G = buf + 3 * kAPart + og;
+    float ad[4] = {0.f, 0.f, 0.f, 0.f}, aa[4] = {0.f, 0.f, 0.f, 0.f};
+    CompSums<2> cd, ca;
+    for (int q = tid; q < n; q += kAConsumers) {
+        const uint4 pw = W[q];
+        const uint4 mw = MOMENTS ? reinterpret_cast<const uint4*>(Mb)[q]
+                                 : words4(reinterpret_cast<const uint32_t*>(Mb) + 4 * q);
+        const uint4 vw = MOMENTS ? reinterpret_cast<const uint4*>(Vb)[q]
+                                 : words4(reinterpret_cast<const uint32_t*>(Vb) + 4 * q);
+        float g[4];
+        if (j.grad_bf16) {
+            uint2 g2;
+            if (LINED) {
+                g2 = reinterpret_cast<const uint2*>(G)[q];
+            } else {
+                const uint32_t* gw = reinterpret_cast<const uint32_t*>(G - (og & 2)) + 2 * q;
+                g2 = make_uint2(gw[0], gw[1]);
+                if (og & 2)
+                    g2 = make_uint2(__funnelshift_r(gw[0], gw[1], 16), __funnelshift_r(gw[1], gw[2], 16));
+            }
+            g[0] = bf16_lo(g2.x); g[1] = bf16_hi(g2.x); g[2] = bf16_lo(g2.y); g[3] = bf16_hi(g2.y);
+        } else {
+            const uint4 g4 = LINED ? reinterpret_cast<const uint4*>(G)[q]
+                                   : words4(reinterpret_cast<const uint32_t*>(G) + 4 * q);
+            g[0] = __uint_as_float(g4.x); g[1] = __uint_as_float(g4.y);
+            g[2] = __uint_as_float(g4.z); g[3] = __uint_as_float(g4.w);
+        }
+        float pv[4] = {__uint_as_float(pw.x), __uint_as_float(pw.y), __uint_as_float(pw.z), __uint_as_float(pw.w)};
+        float m[4] = {__uint_as_float(mw.x), __uint_as_float(mw.y), __uint_as_float(mw.z), __uint_as_float(mw.w)};
+        float v[4] = {__uint_as_float(vw.x), __uint_as_float(vw.y), __uint_as_float(vw.z), __uint_as_float(vw.w)};
+        float pn[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) adam_elem(pv[e], m[e], v[e], g[e], c, pn[e]);
+        if (LINED) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                ad[e] += fabsf(pn[e] - pv[e]);
+                aa[e] += fabsf(pv[e]);
+            }
+        } else {
+            float big = 0.f;                // a NaN is added like any number
+#pragma unroll
+            for (int e = 0; e < 4; ++e) big = fmaxf(big, fmaxf(fabsf(pn[e] - pv[e]), fabsf(pv[e])));
+            const bool fine = big < 1e37f;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                cd.add(e, fine ? fabsf(pn[e] - pv[e]) : 0.f);
+                ca.add(e, fine ? fabsf(pv[e]) : 0.f);
+            }
+            if (!fine) {                    // near the end of fp32's range, or infinite
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    dd += double(fabsf(pn[e] - pv[e]));
+                    da += double(fabsf(pv[e]));
+                }
+            }
+        }
+        const uint4 pnw = make_uint4(__float_as_uint(pn[0]), __float_as_uint(pn[1]), __float_as_uint(pn[2]),
+                                     __float_as_uint(pn[3]));
+        W[q] = pnw;
+        if (MOMENTS) {
+            reinterpret_cast<uint4*>(Mb)[q] = make_uint4(__float_as_uint(m[0]), __float_as_uint(m[1]),
+                                                         __float_as_uint(m[2]), __float_as_uint(m[3]));
+            reinterpret_cast<uint4*>(Vb)[q] = make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]),
+                                                         __float_as_uint(v[2]), __float_as_uint(v[3]));
+        } else {
+            put_words(reinterpret_cast<uint32_t*>(Mb) + 4 * q, j.m, om, q, n, m);
+            put_words(reinterpret_cast<uint32_t*>(Vb) + 4 * q, j.v, ov, q, n, v);
+        }
+        if (j.model) {
+            const uint32_t lo = bf16_pair(pn[0], pn[1]), hi = bf16_pair(pn[2], pn[3]);
+            if (LINED) st_u2(j.model + 8 * q, make_uint2(lo, hi));
+            else put_model(j.model + 8 * q, lo, hi);
+        }
+    }
+    if (LINED) {
+        dd += double((ad[0] + ad[1]) + (ad[2] + ad[3]));
+        da += double((aa[0] + aa[1]) + (aa[2] + aa[3]));
+    } else {
+        cd.reduce();
+        ca.reduce();
+        dd += double(cd.s[0]);
+        da += double(ca.s[0]);
+        ed += cd.e[0];
+        ea += ca.e[0];
     }
 }
 
@@ -366,6 +523,7 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
     const int tid = int(threadIdx.x) - 32 * kAFirstConsumerWarp;
     const int warp = tid >> 5, lane = tid & 31;
     double dd = 0.0, da = 0.0;
+    float ed = 0.f, ea = 0.f;   // rounding errors of the run's compensated chains
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kAStages);
         const uint32_t parity = uint32_t((k / kAStages) & 1);
@@ -379,73 +537,25 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
         mbar_try_wait(full_s + 8 * st, parity);
         const AJob j = r.jobs[st];
         if (j.kind == kAJobEnd) {
-            if (kABulkStore && lane == 0) mbar_arrive(done_s + 8 * st);   // lets the storer see the end
+            if (lane == 0) mbar_arrive(done_s + 8 * st);   // lets the storer see the end
             break;
         }
         if (j.kind == kAJobChunk) {
-            const SegDev sd = p.segs[j.seg];
-            const OptSegDev od = opt[j.seg];
             uint8_t* buf = ring + size_t(st) * kAStage;
-            uint4* W = reinterpret_cast<uint4*>(buf);
-            uint4* M = reinterpret_cast<uint4*>(buf + 16 * kAChunkVec);
-            uint4* V = reinterpret_cast<uint4*>(buf + 32 * kAChunkVec);
-            const uint8_t* G = buf + 48 * kAChunkVec;
-            uint8_t* wb = const_cast<uint8_t*>(sd.w) - 4 * int64_t(sd.lead) + 16 * j.k0;
-            uint8_t* mb = reinterpret_cast<uint8_t*>(od.m) - 4 * int64_t(sd.lead) + 16 * j.k0;
-            uint8_t* vb = reinterpret_cast<uint8_t*>(od.v) - 4 * int64_t(sd.lead) + 16 * j.k0;
-            uint8_t* modb = od.model ? od.model - 2 * int64_t(sd.lead) + 8 * j.k0 : nullptr;
-            const int n = int(j.k1 - j.k0);
-            float ad[4] = {0.f, 0.f, 0.f, 0.f}, aa[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int q = tid; q < n; q += kAConsumers) {
-                const uint4 pw = W[q], mw = M[q], vw = V[q];
-                float g[4];
-                if (od.grad_bf16) {
-                    const uint2 g2 = reinterpret_cast<const uint2*>(G)[q];
-                    g[0] = bf16_lo(g2.x); g[1] = bf16_hi(g2.x); g[2] = bf16_lo(g2.y); g[3] = bf16_hi(g2.y);
-                } else {
-                    const uint4 g4 = reinterpret_cast<const uint4*>(G)[q];
-                    g[0] = __uint_as_float(g4.x); g[1] = __uint_as_float(g4.y);
-                    g[2] = __uint_as_float(g4.z); g[3] = __uint_as_float(g4.w);
-                }
-                float pv[4] = {__uint_as_float(pw.x), __uint_as_float(pw.y), __uint_as_float(pw.z),
-                               __uint_as_float(pw.w)};
-                float m[4] = {__uint_as_float(mw.x), __uint_as_float(mw.y), __uint_as_float(mw.z),
-                              __uint_as_float(mw.w)};
-                float v[4] = {__uint_as_float(vw.x), __uint_as_float(vw.y), __uint_as_float(vw.z),
-                              __uint_as_float(vw.w)};
-                float pn[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    adam_elem(pv[e], m[e], v[e], g[e], c, pn[e]);
-                    ad[e] += fabsf(pn[e] - pv[e]);
-                    aa[e] += fabsf(pv[e]);
-                }
-                const uint4 pnw = make_uint4(__float_as_uint(pn[0]), __float_as_uint(pn[1]),
-                                             __float_as_uint(pn[2]), __float_as_uint(pn[3]));
-                const uint4 mnw = make_uint4(__float_as_uint(m[0]), __float_as_uint(m[1]),
-                                             __float_as_uint(m[2]), __float_as_uint(m[3]));
-                const uint4 vnw = make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]),
-                                             __float_as_uint(v[2]), __float_as_uint(v[3]));
-                if (kABulkStore) {
-                    W[q] = pnw;
-                    M[q] = mnw;
-                    V[q] = vnw;
-                } else {
-                    st_vec(wb + 16 * q, pnw);
-                    st_vec(mb + 16 * q, mnw);
-                    st_vec(vb + 16 * q, vnw);
-                }
-                if (modb) st_u2(modb + 8 * q, make_uint2(bf16_pair(pn[0], pn[1]), bf16_pair(pn[2], pn[3])));
-            }
-            dd += double((ad[0] + ad[1]) + (ad[2] + ad[3]));
-            da += double((aa[0] + aa[1]) + (aa[2] + aa[3]));
+            if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, ed, ea);
+            else if (j.form == kAMoments) adam_chunk<kAMoments>(j, buf, tid, c, dd, da, ed, ea);
+            else adam_chunk<kALoose>(j, buf, tid, c, dd, da, ed, ea);
             // the storer's bulk copies read what this thread wrote to the buffer
-            if (kABulkStore) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         } else if (j.kind == kAJobScalar) {
             const SegDev sd = p.segs[j.seg];
             const OptSegDev od = opt[j.seg];
             for (int64_t q = j.k0 + tid; q < j.k1; q += kAConsumers) adam_scalar_vector(sd, od, q, c, dd, da);
         } else {
+            dd += double(ed);
+            da += double(ea);
+            ed = 0.f;
+            ea = 0.f;
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) {
                 dd += __shfl_down_sync(0xffffffffu, dd, off);
@@ -456,14 +566,22 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             da = 0.0;
         }
         __syncwarp();
-        if (lane == 0) mbar_arrive((kABulkStore ? done_s : empty_s) + 8 * st);
+        if (lane == 0) mbar_arrive(done_s + 8 * st);
     }
 }
 
-// Bulk-store form: once every consumer warp is done with a buffer, write its
+// The whole granules of n vectors that start at `first`, staged from the
+// granule below it on.
+__device__ __forceinline__ void put_granules(uint8_t* first, uint32_t staged, uint32_t n) {
+    const uint32_t off = uint32_t(uintptr_t(first) & 15);
+    if (off == 0) bulk_s2g(first, staged, 16 * n);
+    else if (n > 1) bulk_s2g(first - off + 16, staged + 16, 16 * (n - 1));
+}
+
+// Once every consumer warp is done with a buffer, write its
 // updated w, m and v back with bulk stores, and hand the buffer to the
 // producer when those stores have read it.
-__device__ void adam_store(const MeasureParams& p, const OptSegDev* opt, const uint8_t* ring, ARing& r) {
+__device__ void adam_store(const MeasureParams& p, const uint8_t* ring, ARing& r) {
     const uint32_t done_s = smem_addr(r.computed), empty_s = smem_addr(r.empty);
     const uint32_t ring_s = smem_addr(ring);
     for (uint64_t k = 0;; ++k) {
@@ -475,22 +593,11 @@ __device__ void adam_store(const MeasureParams& p, const OptSegDev* opt, const u
         const AJob j = r.jobs[st];
         if (j.kind == kAJobEnd) break;
         if (j.kind == kAJobChunk) {
-            const SegDev sd = p.segs[j.seg];
-            const OptSegDev od = opt[j.seg];
-            const int64_t off = 16 * j.k0 - 4 * int64_t(sd.lead);
-            const uint32_t bytes = uint32_t(j.k1 - j.k0) * 16u;
+            const uint32_t n = uint32_t(j.n);
             const uint32_t buf = ring_s + uint32_t(st) * kAStage;
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(sd.w + off),
-                         "r"(buf), "r"(bytes)
-                         : "memory");
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                             reinterpret_cast<uint8_t*>(od.m) + off),
-                         "r"(buf + 16 * kAChunkVec), "r"(bytes)
-                         : "memory");
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
-                             reinterpret_cast<uint8_t*>(od.v) + off),
-                         "r"(buf + 32 * kAChunkVec), "r"(bytes)
-                         : "memory");
+            bulk_s2g(j.w, buf, 16 * n);
+            put_granules(j.m, buf + kAPart, n);
+            put_granules(j.v, buf + 2 * kAPart, n);
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
@@ -509,7 +616,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
         for (int st = 0; st < kAStages; ++st) {
             mbar_init(smem_addr(&r.full[st]), 1);
             mbar_init(smem_addr(&r.computed[st]), kAConsumerWarps);
-            mbar_init(smem_addr(&r.empty[st]), kABulkStore ? 1 : kAConsumerWarps);
+            mbar_init(smem_addr(&r.empty[st]), 1);
             r.box.count[st] = 0u;
         }
         mbar_init_fence();
@@ -517,8 +624,8 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
     __syncthreads();
     if (threadIdx.x == 0) {
         adam_produce(p, opt, ring, r);
-    } else if (kABulkStore && threadIdx.x < 64) {
-        if (threadIdx.x == 32) adam_store(p, opt, ring, r);
+    } else if (threadIdx.x < 64) {
+        if (threadIdx.x == 32) adam_store(p, ring, r);
     } else if (threadIdx.x >= 32) {
         adam_consume(p, opt, c, ring, r);
     }

@@ -74,6 +74,12 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src, uin
         : "memory");
 }
 
+// shared -> global, in the thread's current bulk group.
+__device__ __forceinline__ void bulk_s2g(void* dst, uint32_t src_smem, uint32_t bytes) {
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src_smem), "r"(bytes)
+                 : "memory");
+}
+
 // Bytes [SH, SH + 16) of the 32 bytes of a and b (SH even).
 template <int SH>
 __device__ __forceinline__ uint4 window16(const uint4& a, const uint4& b) {

@@ -333,49 +333,6 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
     }
 }
 
-// a + b, its rounding error added to e (exact in any order of magnitude).
-__device__ __forceinline__ float two_sum(float a, float b, float& e) {
-    const float s = a + b, t = s - a;
-    e += (a - (s - t)) + (b - t);
-    return s;
-}
-
-// The same in three operations: exact once the sum a is at least as large as
-// the term b; before that within half the error that plain addition makes.
-__device__ __forceinline__ float fast_two_sum(float a, float b, float& e) {
-    const float s = a + b;
-    e += b - (s - a);
-    return s;
-}
-
-// One chunk's fp32 chains of a thread with their rounding errors.  bf16
-// terms have 8 significant bits, so a chain rounds only where two terms are
-// more than 2^16 apart and the short form serves; fp32 terms round in every
-// addition and there are half as many of them per byte.
-template <int ESZ_LOG2>
-struct CompSums {
-    static constexpr int kLanes = 16 >> ESZ_LOG2;
-    float s[kLanes], e[kLanes];
-    __device__ __forceinline__ CompSums() {
-#pragma unroll
-        for (int i = 0; i < kLanes; ++i) { s[i] = 0.f; e[i] = 0.f; }
-    }
-    __device__ __forceinline__ void add(int i, float x) {
-        s[i] = ESZ_LOG2 == 1 ? fast_two_sum(s[i], x, e[i]) : two_sum(s[i], x, e[i]);
-    }
-    // the chains' sum, left in s[0] and e[0]
-    __device__ __forceinline__ void reduce() {
-#pragma unroll
-        for (int k = kLanes / 2; k > 0; k >>= 1) {
-#pragma unroll
-            for (int i = 0; i < k; ++i) {
-                e[i] += e[i + k];
-                s[i] = two_sum(s[i], s[i + k], e[i]);
-            }
-        }
-    }
-};
-
 template <int ESZ_LOG2>
 __device__ __forceinline__ void accumulate_comp(const uint4& w, const uint4& r, CompSums<ESZ_LOG2>& cd,
                                                 CompSums<ESZ_LOG2>& ca) {

@@ -1,7 +1,8 @@
 // lc_reduce.cuh -- device helpers shared by the kernels that reduce over
 // the measure work space (lc_measure.cu: the Eq. 1 scan; lc_adamw.cu: the
 // fused optimizer step): streaming loads and stores, bf16 decoding, the
-// fixed-order CTA sum and the last-CTA fp64 combine per segment and layer.
+// fixed-order CTA sum and the last-CTA fp64 combine per segment and layer,
+// and fp32 chains that keep their rounding errors.
 #pragma once
 
 #include "lc_internal.cuh"
@@ -46,6 +47,49 @@ __device__ __forceinline__ void st_vec(void* p, uint4 v) {
 
 __device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
+
+// a + b, its rounding error added to e (exact in any order of magnitude).
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+    const float s = a + b, t = s - a;
+    e += (a - (s - t)) + (b - t);
+    return s;
+}
+
+// The same in three operations: exact once the sum a is at least as large as
+// the term b; before that within half the error that plain addition makes.
+__device__ __forceinline__ float fast_two_sum(float a, float b, float& e) {
+    const float s = a + b;
+    e += b - (s - a);
+    return s;
+}
+
+// One chunk's fp32 chains of a thread with their rounding errors.  bf16
+// terms have 8 significant bits, so a chain rounds only where two terms are
+// more than 2^16 apart and the short form serves; fp32 terms round in every
+// addition and there are half as many of them per byte.
+template <int ESZ_LOG2>
+struct CompSums {
+    static constexpr int kLanes = 16 >> ESZ_LOG2;
+    float s[kLanes], e[kLanes];
+    __device__ __forceinline__ CompSums() {
+#pragma unroll
+        for (int i = 0; i < kLanes; ++i) { s[i] = 0.f; e[i] = 0.f; }
+    }
+    __device__ __forceinline__ void add(int i, float x) {
+        s[i] = ESZ_LOG2 == 1 ? fast_two_sum(s[i], x, e[i]) : two_sum(s[i], x, e[i]);
+    }
+    // the chains' sum, left in s[0] and e[0]
+    __device__ __forceinline__ void reduce() {
+#pragma unroll
+        for (int k = kLanes / 2; k > 0; k >>= 1) {
+#pragma unroll
+            for (int i = 0; i < k; ++i) {
+                e[i] += e[i + k];
+                s[i] = two_sum(s[i], s[i + k], e[i]);
+            }
+        }
+    }
+};
 
 // Sum over the CTA in a fixed order; the result is valid in thread 0.
 __device__ __forceinline__ void block_sum(double& d, double& a, double* sd, double* sa) {

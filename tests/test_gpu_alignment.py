@@ -174,3 +174,63 @@ def test_pack_commit_restore_off_alignment(dtype, fuse, staging):
         for buf, view, o in part:
             assert set(_outside(buf, view, o)) == {0xA5}, "bytes beside a tensor were written"
     lc.close()
+
+
+@pytest.mark.parametrize("grad_dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("lead", [0, 8])
+def test_adamw_off_alignment(lead, grad_dtype):
+    """The fused step with moments, gradients and model copies at every
+    offset from the weights' vectors: each array equals the step's fp32
+    operations done one by one on the CPU, bit for bit, and nothing beside
+    it is written.  The sums are within the roundings of a chunk's chains
+    (three terms and a tree of four) of the 64-bit ones."""
+    torch = require_gpu()
+    import paper_2609_27193_gb300 as P
+    gt = torch.bfloat16 if grad_dtype == "bf16" else torch.float32
+    gsz = 2 if grad_dtype == "bf16" else 4
+    g = torch.Generator().manual_seed(lead + gsz)
+    hp = dict(lr=1e-3, beta1=0.9, beta2=0.95, eps=1e-8, weight_decay=0.1)
+    sizes = [1, 2, 3, 4, 5, 8, 9, 11, 31, 257, 2047, 2048, 2049, 4100, 100003]
+    combos = [(4 * (k % 4), 4 * (k // 4 % 4), gsz * (k % (16 // gsz)), 2 * ((3 * k + 1) % 8)) for k in range(16)]
+    segs, keep, grads, models = [], [], [], []
+    for k, (om, ov, og, oc) in enumerate(combos):
+        for n in sizes:
+            p = torch.randn(n, generator=g) * 0.02
+            m = torch.randn(n, generator=g) * 1e-3
+            v = torch.randn(n, generator=g).abs() * 1e-6
+            x = (torch.randn(n, generator=g) * 1e-3).to(gt)
+            part = [_placed(torch, n, d, o) + (o,) for d, o in
+                    ((torch.float32, lead), (torch.float32, om), (torch.float32, ov), (gt, og), (torch.bfloat16, oc))]
+            for t, src in zip(part, (p, m, v, x)):
+                t[1].copy_(src)
+            keep.append((part, p, m, v, x))
+            segs.append(P.segment(k, part[0][1], None, part[1][1], part[2][1]))
+            grads.append(part[3][1])
+            models.append(part[4][1])
+    N = len(combos)
+    lc = P.LayerCheck(mode=P.LC_DRIFT_ACCUMULATE)
+    lc.register_layout(segs, N)
+    lc.register_optimizer(grads, models)
+    sums = torch.zeros(3 * N, dtype=torch.float64, device="cuda")
+    lc.set_layer_sums_buffer(sums)
+    lc.adamw_step_measure(1, **hp)
+    torch.cuda.synchronize()
+    f = lambda x: torch.tensor(np.float32(x))
+    want = np.zeros((N, 3))
+    for s, (part, p, m, v, x) in zip(segs, keep):
+        x = x.float()
+        m2 = m * f(0.9) + x * f(1 - 0.9)
+        v2 = v * f(0.95) + (x * x) * f(1 - 0.95)
+        vh = v2 * f(1 / (1 - 0.95))
+        p2 = p * f(1 - 1e-3 * 0.1) - (m2 * f(1e-3 / (1 - 0.9))) / (torch.sqrt(vh) + f(1e-8))
+        want[s.layer] += ((p2 - p).abs().double().sum().item(), p.abs().double().sum().item(), p.numel())
+        for t, ref in zip((part[0], part[1], part[2]), (p2, m2, v2)):
+            assert torch.equal(t[1].cpu().view(torch.int32), ref.view(torch.int32)), (s.layer, p.numel())
+        assert torch.equal(part[4][1].cpu().view(torch.int16), p2.to(torch.bfloat16).view(torch.int16))
+        for buf, view, o in part:
+            assert set(_outside(buf, view, o)) == {0xA5}, "bytes beside an array were written"
+    got = sums.cpu().numpy().reshape(N, 3)
+    assert np.array_equal(got[:, 2], want[:, 2])
+    assert (np.abs(got - want) <= 5 * 2.0 ** -24 * np.abs(want)).all()
+    assert lc.counters()["bulk_measure_launches"] == 1
+    lc.close()
