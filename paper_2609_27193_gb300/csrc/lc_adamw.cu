@@ -190,19 +190,22 @@ __global__ void __launch_bounds__(kMeasureThreads, LC_ADAM_MIN_BLOCKS) adamw_mea
     const int64_t v1 = p.cta_vec_begin[b + 1];
     int s = p.cta_seg0[b];
     int slot = p.cta_slot0[b];
+    double dd = 0.0, da = 0.0;
     while (v0 < v1 && s < p.nseg) {
         const SegDev sd = p.segs[s];
         const OptSegDev od = opt[s];
         const int64_t seg_end = sd.vec_begin + sd.nvec;
         const int64_t lo = v0 - sd.vec_begin;
         const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
-        double dd = 0.0, da = 0.0;
         adam_run(sd, od, lo, hi, c, dd, da);
+        ++s;
+        v0 = sd.vec_begin + hi;
+        if (v0 < v1 && s < p.nseg && p.segs[s].layer == sd.layer) continue;
         block_sum(dd, da, red_d, red_a);
         if (threadIdx.x == 0) p.partials[slot] = make_double2(dd, da);
         ++slot;
-        ++s;
-        v0 = sd.vec_begin + hi;
+        dd = 0.0;
+        da = 0.0;
     }
     if (threadIdx.x == 0) {
         __threadfence();
@@ -351,12 +354,23 @@ __device__ void adam_produce(const MeasureParams& p, const OptSegDev* opt, uint8
         const int64_t v1 = p.cta_vec_begin[rng + 1];
         int s = p.cta_seg0[rng];
         int slot = p.cta_slot0[rng];
-        while (ok && v0 < v1 && s < p.nseg) {
+        if (v0 < v1 && s < p.nseg) {
             sd = p.segs[s];
             od = opt[s];
+        }
+        while (ok && v0 < v1 && s < p.nseg) {
             const int64_t seg_end = sd.vec_begin + sd.nvec;
             const int64_t lo = v0 - sd.vec_begin;
             const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
+            // the next segment is fetched while this one streams; the run ends with its layer
+            SegDev next;
+            OptSegDev onext;
+            const bool more = seg_end < v1 && s + 1 < p.nseg;
+            if (more) {
+                next = p.segs[s + 1];
+                onext = opt[s + 1];
+            }
+            const bool run_ends = !more || next.layer != sd.layer;
             // vectors [kf0, kf1) lie inside w with their windows inside m, v and the gradient
             int64_t kf0 = sd.lead > 0 ? 1 : 0;
             int64_t kf1 = (int64_t(sd.lead) + sd.numel) / 4;
@@ -369,10 +383,11 @@ __device__ void adam_produce(const MeasureParams& p, const OptSegDev* opt, uint8
             for (int64_t x = lo > kf0 ? lo : kf0; ok && x < e; x += kAChunkVec)
                 ok = post(kAJobChunk, s, slot, x, (x + kAChunkVec < e ? x + kAChunkVec : e));
             if (ok && hi > kf1) ok = post(kAJobScalar, s, slot, (lo > kf1 ? lo : kf1), hi);
-            if (ok) ok = post(kAJobFlush, s, slot, 0, 0);
-            slot += kMeasureBulkSlotsPerRun;
+            if (ok && run_ends) ok = post(kAJobFlush, s, slot++, 0, 0);
             ++s;
             v0 = sd.vec_begin + hi;
+            sd = next;
+            od = onext;
         }
     }
     if (ok) ok = post(kAJobEnd, 0, 0, 0, 0);
@@ -423,7 +438,7 @@ __device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi)
 // element and takes 1885 (floor 1696 at 6.8 TB/s).
 template <int FORM>
 __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid, const AdamConsts& c, double& dd,
-                                           double& da, float& ed, float& ea) {
+                                           double& da, float& ed, float& ea, float& td, float& ta) {
     constexpr bool LINED = FORM == kALined, MOMENTS = FORM != kALoose;
     const int n = j.n;
     uint4* W = reinterpret_cast<uint4*>(buf);
@@ -507,13 +522,13 @@ __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid,
         }
     }
     if (LINED) {
-        dd += double((ad[0] + ad[1]) + (ad[2] + ad[3]));
-        da += double((aa[0] + aa[1]) + (aa[2] + aa[3]));
+        td = (ad[0] + ad[1]) + (ad[2] + ad[3]);
+        ta = (aa[0] + aa[1]) + (aa[2] + aa[3]);
     } else {
         cd.reduce();
         ca.reduce();
-        dd += double(cd.s[0]);
-        da += double(ca.s[0]);
+        td = cd.s[0];
+        ta = ca.s[0];
         ed += cd.e[0];
         ea += ca.e[0];
     }
@@ -530,24 +545,21 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kAStages);
         const uint32_t parity = uint32_t((k / kAStages) & 1);
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait_bounded(full_s + 8 * st, parity, kWaitNs) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
+        if (!mbar_wait_warp(full_s + 8 * st, parity)) {
             if (lane == 0) raise_fault(p.fault);
             break;
         }
-        mbar_try_wait(full_s + 8 * st, parity);
         const AJob j = r.jobs[st];
         if (j.kind == kAJobEnd) {
             if (lane == 0) mbar_arrive(done_s + 8 * st);   // lets the storer see the end
             break;
         }
+        float td = 0.f, ta = 0.f;   // the chunk's sums
         if (j.kind == kAJobChunk) {
             uint8_t* buf = ring + size_t(st) * kAStage;
-            if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, ed, ea);
-            else if (j.form == kAMoments) adam_chunk<kAMoments>(j, buf, tid, c, dd, da, ed, ea);
-            else adam_chunk<kALoose>(j, buf, tid, c, dd, da, ed, ea);
+            if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, ed, ea, td, ta);
+            else if (j.form == kAMoments) adam_chunk<kAMoments>(j, buf, tid, c, dd, da, ed, ea, td, ta);
+            else adam_chunk<kALoose>(j, buf, tid, c, dd, da, ed, ea, td, ta);
             // the storer's bulk copies read what this thread wrote to the buffer
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         } else if (j.kind == kAJobScalar) {
@@ -559,17 +571,14 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             da += double(ea);
             ed = 0.f;
             ea = 0.f;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                dd += __shfl_down_sync(0xffffffffu, dd, off);
-                da += __shfl_down_sync(0xffffffffu, da, off);
-            }
-            if (lane == 0) run_box_put<kAConsumerWarps>(r.box, st, warp, dd, da, p.partials + j.slot);
+            run_flush<kAConsumerWarps>(r.box, st, warp, lane, dd, da, p.partials + j.slot);
             dd = 0.0;
             da = 0.0;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(done_s + 8 * st);
+        mbar_arrive_warp(done_s + 8 * st, lane);
+        after_handback(td, ta);
+        dd += double(td);
+        da += double(ta);
     }
 }
 
@@ -615,6 +624,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
     extern __shared__ __align__(128) uint8_t ring[];
     __shared__ __align__(8) ARing r;
     __shared__ unsigned int s_ticket;
+    __shared__ __align__(8) FinTables tables;
     if (threadIdx.x == 0) {
         for (int st = 0; st < kAStages; ++st) {
             mbar_init(smem_addr(&r.full[st]), 1);
@@ -624,6 +634,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
         }
         mbar_init_fence();
     }
+    fin_prefetch(p, tables);
     __syncthreads();
     if (threadIdx.x == 0) {
         adam_produce(p, opt, ring, r);
@@ -632,6 +643,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
     } else if (threadIdx.x >= 32) {
         adam_consume(p, opt, c, ring, r);
     }
+    fin_prefetch_wait();
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -641,7 +653,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
     if (s_ticket != gridDim.x - 1) return;
     __threadfence();
     // every load and bulk store of the ring is complete: it stages the combine
-    finalize(p, reinterpret_cast<double2*>(ring), int32_t(kAdamBulkSmem / sizeof(double2)));
+    finalize(p, reinterpret_cast<double2*>(ring), int32_t(kAdamBulkSmem / sizeof(double2)), &tables);
 }
 
 }  // namespace

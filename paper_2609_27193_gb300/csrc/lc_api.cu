@@ -45,6 +45,9 @@ using namespace lc;
 #ifndef LC_MEASURE_POOL_PCT
 #define LC_MEASURE_POOL_PCT 10
 #endif
+#ifndef LC_MEASURE_POOL_MIN
+#define LC_MEASURE_POOL_MIN 1024
+#endif
 #ifndef LC_MEASURE_POOL_UNITS
 #define LC_MEASURE_POOL_UNITS 8
 #endif
@@ -793,18 +796,17 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         V += d.nvec;
     }
     // CTA work ranges of the measure work space: G equal shares in granules
-    // of LC_MEASURE_ALIGN_VECS, and `per_run` partial slots for every
-    // (CTA, segment) run
+    // of LC_MEASURE_ALIGN_VECS, and a partial slot for every (range, layer) run
     // (with a pool: G static ranges over the first granules, then `units`
     // ranges over the rest; range r's slots are fixed whichever CTA walks it)
     struct Partition {
         int64_t G = 0;
         int64_t units = 0;
         std::vector<int64_t> cta_vec;
-        std::vector<int32_t> cta_seg0, cta_slot0, seg_slot_begin;
+        std::vector<int32_t> cta_seg0, cta_slot0, layer_slot_begin;
         int32_t nslots = 0;
     };
-    auto partition = [&](int64_t grid, int32_t per_run, int64_t pool_pct = 0, int64_t units_per_cta = 0) {
+    auto partition = [&](int64_t grid, int64_t pool_pct = 0, int64_t units_per_cta = 0) {
         Partition pt;
         const int64_t gran = LC_MEASURE_ALIGN_VECS;
         const int64_t ngran = (V + gran - 1) / gran;
@@ -813,7 +815,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         // granules in the pool, in units of at least kMinUnit granules (512 KB
         // of W: a unit costs a counter fetch, a table lookup and a flush); a
         // pool too small to give every CTA a unit on average is not used
-        constexpr int64_t kMinUnit = 1024;
+        constexpr int64_t kMinUnit = LC_MEASURE_POOL_MIN;
         int64_t pool = pool_pct > 0 ? ngran * pool_pct / 100 : 0;
         pt.units = pool >= G * kMinUnit ? std::min<int64_t>(G * units_per_cta, pool / kMinUnit) : 0;
         if (pt.units == 0) pool = 0;
@@ -821,7 +823,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         pt.cta_vec.resize(R + 1);
         pt.cta_seg0.resize(R);
         pt.cta_slot0.resize(R);
-        pt.seg_slot_begin.assign(nseg + 1, -1);
+        pt.layer_slot_begin.assign(nlayers + 1, -1);
         for (int64_t b = 0; b <= G; ++b) pt.cta_vec[b] = std::min(V, ng_static * b / G * gran);
         for (int64_t u = 1; u <= U; ++u) pt.cta_vec[G + u] = std::min(V, (ng_static + pool * u / U) * gran);
         int32_t slot = 0, s = 0;
@@ -830,24 +832,28 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
             while (s < nseg && sd[s].vec_begin + sd[s].nvec <= v0) ++s;
             pt.cta_seg0[b] = s;
             pt.cta_slot0[b] = slot;
+            // one slot per layer of the range; ranges and layers both follow
+            // the work space, so a layer's slots are contiguous
             for (int32_t t = s; v0 < v1 && t < nseg && sd[t].vec_begin < v1; ++t) {
-                if (pt.seg_slot_begin[t] < 0) pt.seg_slot_begin[t] = slot;
-                slot += per_run;
+                if (t > s && sd[t].layer == sd[t - 1].layer) continue;
+                int32_t& first = pt.layer_slot_begin[sd[t].layer];
+                if (first < 0) first = slot;
+                ++slot;
             }
         }
-        pt.seg_slot_begin[nseg] = slot;
-        for (int32_t t = nseg - 1; t >= 0; --t)
-            if (pt.seg_slot_begin[t] < 0) pt.seg_slot_begin[t] = pt.seg_slot_begin[t + 1];
+        pt.layer_slot_begin[nlayers] = slot;
+        for (int32_t l = nlayers - 1; l >= 0; --l)
+            if (pt.layer_slot_begin[l] < 0) pt.layer_slot_begin[l] = pt.layer_slot_begin[l + 1];
         pt.nslots = slot;
         return pt;
     };
     int occ = 0;
     LC_CUDA(measure_occupancy(&occ));
-    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ), 1);
+    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ));
     int bocc = 0;
     LC_CUDA(measure_bulk_prepare(&bocc));
     const Partition pb = partition(int64_t(ctx->sms) * std::max(1, bocc) * LC_MEASURE_BULK_WAVES,
-                                   kMeasureBulkSlotsPerRun, LC_MEASURE_POOL_PCT, LC_MEASURE_POOL_UNITS);
+                                   LC_MEASURE_POOL_PCT, LC_MEASURE_POOL_UNITS);
     const int64_t Rb = pb.G + pb.units;
     const int64_t G = pa.G, Gb = pb.G;
     ctx->measure_grid = int(G);
@@ -909,17 +915,16 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     const size_t o_ctav = tp.take(sizeof(int64_t) * (G + 1));
     const size_t o_ctas = tp.take(sizeof(int32_t) * G);
     const size_t o_ctal = tp.take(sizeof(int32_t) * G);
-    const size_t o_segslot = tp.take(sizeof(int32_t) * (nseg + 1));
-    const size_t o_lsb = tp.take(sizeof(int32_t) * (nlayers + 1));
+    const size_t o_lslot = tp.take(sizeof(int32_t) * (nlayers + 1));
+    const size_t o_ln = tp.take(sizeof(double) * nlayers);
     const size_t o_part = tp.take(sizeof(double2) * std::max(1, ctx->nslots));
-    const size_t o_segsum = tp.take(sizeof(double) * 2 * nseg);
     const size_t o_sums = tp.take(sizeof(double) * 3 * nlayers);
     const size_t o_ticket = tp.take(sizeof(unsigned int));
     const size_t o_ctav_b = tp.take(sizeof(int64_t) * (Rb + 1));
     const size_t o_ctas_b = tp.take(sizeof(int32_t) * Rb);
     const size_t o_ctal_b = tp.take(sizeof(int32_t) * Rb);
     const size_t o_unit_b = tp.take(sizeof(unsigned int));
-    const size_t o_segslot_b = tp.take(sizeof(int32_t) * (nseg + 1));
+    const size_t o_lslot_b = tp.take(sizeof(int32_t) * (nlayers + 1));
     const size_t o_part_b = tp.take(sizeof(double2) * std::max(1, pb.nslots));
     const size_t o_ticket_b = tp.take(sizeof(unsigned int));
     const size_t o_delta = tp.take(sizeof(double) * nlayers);
@@ -952,12 +957,13 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     put(o_ctav, pa.cta_vec.data(), sizeof(int64_t) * (G + 1));
     put(o_ctas, pa.cta_seg0.data(), sizeof(int32_t) * G);
     put(o_ctal, pa.cta_slot0.data(), sizeof(int32_t) * G);
-    put(o_segslot, pa.seg_slot_begin.data(), sizeof(int32_t) * (nseg + 1));
+    put(o_lslot, pa.layer_slot_begin.data(), sizeof(int32_t) * (nlayers + 1));
     put(o_ctav_b, pb.cta_vec.data(), sizeof(int64_t) * (Rb + 1));
     put(o_ctas_b, pb.cta_seg0.data(), sizeof(int32_t) * Rb);
     put(o_ctal_b, pb.cta_slot0.data(), sizeof(int32_t) * Rb);
-    put(o_segslot_b, pb.seg_slot_begin.data(), sizeof(int32_t) * (nseg + 1));
-    put(o_lsb, ctx->layer_seg_begin.data(), sizeof(int32_t) * (nlayers + 1));
+    put(o_lslot_b, pb.layer_slot_begin.data(), sizeof(int32_t) * (nlayers + 1));
+    const std::vector<double> layer_n(ctx->layer_numel.begin(), ctx->layer_numel.end());
+    put(o_ln, layer_n.data(), sizeof(double) * nlayers);
     put(o_mult, mult.data(), sizeof(double) * nlayers);
     put(o_lnumel, ctx->layer_numel.data(), sizeof(int64_t) * nlayers);
     put(o_lbytes, ctx->layer_bytes.data(), sizeof(uint64_t) * nlayers);
@@ -978,10 +984,9 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     mp.cta_vec_begin = reinterpret_cast<const int64_t*>(base + o_ctav);
     mp.cta_seg0 = reinterpret_cast<const int32_t*>(base + o_ctas);
     mp.cta_slot0 = reinterpret_cast<const int32_t*>(base + o_ctal);
-    mp.seg_slot_begin = reinterpret_cast<const int32_t*>(base + o_segslot);
-    mp.layer_seg_begin = reinterpret_cast<const int32_t*>(base + o_lsb);
+    mp.layer_slot_begin = reinterpret_cast<const int32_t*>(base + o_lslot);
+    mp.layer_n = reinterpret_cast<const double*>(base + o_ln);
     mp.partials = reinterpret_cast<double2*>(base + o_part);
-    mp.seg_sums = reinterpret_cast<double*>(base + o_segsum);
     mp.sums = reinterpret_cast<double*>(base + o_sums);
     mp.ticket = reinterpret_cast<unsigned int*>(base + o_ticket);
     mp.nseg = nseg;
@@ -993,7 +998,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     mpb.cta_vec_begin = reinterpret_cast<const int64_t*>(base + o_ctav_b);
     mpb.cta_seg0 = reinterpret_cast<const int32_t*>(base + o_ctas_b);
     mpb.cta_slot0 = reinterpret_cast<const int32_t*>(base + o_ctal_b);
-    mpb.seg_slot_begin = reinterpret_cast<const int32_t*>(base + o_segslot_b);
+    mpb.layer_slot_begin = reinterpret_cast<const int32_t*>(base + o_lslot_b);
     mpb.partials = reinterpret_cast<double2*>(base + o_part_b);
     mpb.ticket = reinterpret_cast<unsigned int*>(base + o_ticket_b);
     mpb.units = int32_t(pb.units);

@@ -47,13 +47,38 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
 }
 
 // Waits for the phase with the given parity to complete, for at most
-// `limit_ns` (and kWaitIters polls).  Returns false if it gave up.
-__device__ __noinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
+// `limit_ns` (and kWaitIters polls).  Returns false if it gave up.  A poll
+// suspends the thread for a while in hardware; the timer is read on every
+// kPollsPerTime-th one only.
+constexpr uint32_t kPollsPerTime = 16;
+__device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t parity, uint64_t limit_ns) {
     if (mbar_try_wait(bar, parity)) return true;
-    const uint64_t t0 = global_ns();
-    for (uint32_t it = 0; it < kWaitIters; ++it) {
+    uint64_t t0 = 0;
+    for (uint32_t it = 1; it < kWaitIters; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
-        if (global_ns() - t0 > limit_ns) return false;
+        if (it % kPollsPerTime) continue;
+        const uint64_t t = global_ns();
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > limit_ns) return false;
+    }
+    return false;
+}
+
+// A consumer warp's wait: its lanes poll together and take the outcome
+// together.  True: the phase is complete and every lane's reads come after
+// it.  (With lane 0 polling for the warp, unrelated code in the loop decided
+// between two speeds of the whole kernel: the 8B measure took 4.28 or 4.79 ms,
+// the fused step over 1.2 G parameters 5.22 or 6.66 ms.  This way it has been
+// the faster one with every variant of that code.)
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    uint64_t t0 = 0;
+    for (uint32_t it = 1; it < kWaitIters; ++it) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (it % kPollsPerTime) continue;
+        const uint64_t t = __shfl_sync(0xffffffffu, global_ns(), 0);
+        if (t0 == 0) t0 = t;
+        else if (t - t0 > kWaitNs) return false;
     }
     return false;
 }
@@ -65,6 +90,19 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+
+// One arrival for the warp, once all its lanes are done.  What the warp still
+// does with registers alone comes after it (after_handback): the buffer's next
+// load then starts before that work, not behind it.
+__device__ __forceinline__ void mbar_arrive_warp(uint32_t bar, int lane) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+    __syncwarp();
+}
+
+// Keeps the use of x and y behind the hand-back that precedes it: arithmetic on
+// registers may otherwise be scheduled ahead of it.
+__device__ __forceinline__ void after_handback(float& x, float& y) { asm volatile("" : "+f"(x), "+f"(y)::"memory"); }
 
 // global -> shared, completing `bytes` of the barrier's transaction count.
 __device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src, uint32_t bytes, uint32_t bar) {

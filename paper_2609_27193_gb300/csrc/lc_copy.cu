@@ -589,21 +589,16 @@ __device__ void shift_consume(const CopyParams& p, const uint8_t* ring, ShiftRin
     for (uint64_t k = 0;; ++k) {
         const int s = int(k % kStages);
         const uint32_t parity = uint32_t((k / kStages) & 1);
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait_bounded(full_s + 8 * s, parity, kWaitNs) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
+        if (!mbar_wait_warp(full_s + 8 * s, parity)) {
             if (lane == 0) raise_copy_fault(p);
             break;
         }
-        mbar_try_wait(full_s + 8 * s, parity);   // completed: orders this lane's reads after the loads
         const ShiftJob j = r.jobs[s];
         if (j.bytes == 0) break;
         const uint8_t* staged = ring + size_t(s) * kChunk;
         put_staged(staged, j.bytes, j.dst, tid);
         if (j.dst2) put_staged(staged, j.bytes, j.dst2, tid);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty_s + 8 * s);
+        mbar_arrive_warp(empty_s + 8 * s, lane);
     }
 }
 

@@ -44,10 +44,9 @@ struct MeasureParams {
     const int64_t* cta_vec_begin;    // [G+1] vector range of every CTA
     const int32_t* cta_seg0;         // [G]   first segment each CTA touches
     const int32_t* cta_slot0;        // [G]   first partial slot of each CTA
-    const int32_t* seg_slot_begin;   // [nseg+1] slots of segment s: [begin[s], begin[s+1])
-    const int32_t* layer_seg_begin;  // [nlayers+1] segments of layer l
-    double2* partials;               // [nslots] (sum|W-R|, sum|R|) per (CTA, segment) run
-    double* seg_sums;                // [2*nseg]  per-segment (D, A)
+    const int32_t* layer_slot_begin; // [nlayers+1] slots of layer l: [begin[l], begin[l+1])
+    const double* layer_n;           // [nlayers] elements of layer l
+    double2* partials;               // [nslots] (sum|W-R|, sum|R|) per (range, layer) run
     double* sums;                    // [3*nlayers] per-layer (D, A, n)
     unsigned int* ticket;            // CTA completion counter (reset by the last CTA)
     int32_t nseg;
@@ -204,17 +203,15 @@ struct AdamConsts {
 cudaError_t launch_measure(const MeasureParams& p, int grid, bool write_ref, cudaStream_t s);
 cudaError_t measure_occupancy(int* blocks_per_sm);
 // Bulk-load measure: W and R stream through a shared-memory ring
-// (cp.async.bulk); its partition gives every (CTA, segment) run
-// kMeasureBulkSlotsPerRun partial slots (the CTA's consumer warps combine
-// their shares into one).  W and R must be device memory.  write_ref:
-// accumulate mode (R <- W as well).
-constexpr int kMeasureBulkSlotsPerRun = 1;
+// (cp.async.bulk); the CTA's consumer warps combine their shares of a run
+// into its slot.  W and R must be device memory.  write_ref: accumulate mode
+// (R <- W as well).
 cudaError_t launch_measure_bulk(const MeasureParams& p, int grid, bool write_ref, cudaStream_t s);
 cudaError_t measure_bulk_prepare(int* blocks_per_sm);
 cudaError_t launch_adamw_measure(const MeasureParams& p, const OptSegDev* opt, const AdamConsts& c,
                                  int grid, cudaStream_t s);
 // The fused step with its loads on the bulk engine: the bulk-load measure's
-// partition (kMeasureBulkSlotsPerRun slots per run); every array device memory.
+// partition; every array device memory.
 cudaError_t launch_adamw_bulk(const MeasureParams& p, const OptSegDev* opt, const AdamConsts& c, int grid,
                               cudaStream_t s);
 cudaError_t adamw_bulk_prepare(int* blocks_per_sm);

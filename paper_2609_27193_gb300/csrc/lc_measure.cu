@@ -1,5 +1,5 @@
-// lc_measure.cu -- Eq. 1 (§3.2) on sm_103a: per segment sum|W - R| and
-// sum|R|, combined per layer with the element count.
+// lc_measure.cu -- Eq. 1 (§3.2) on sm_103a: per layer sum|W - R|, sum|R| and
+// the element count.
 //
 // Work decomposition: every segment is covered by 16-byte "virtual vectors"
 // aligned to absolute addresses (lc_internal.cuh).  All vectors of all
@@ -8,10 +8,9 @@
 // the device (one wave), and for the bulk kernel a pool of small ones after
 // them.  A CTA streams its range(s) (the thread kernel: 128-bit
 // non-allocating loads of W and R, several in flight per thread) and writes
-// one fp64 partial per (range, segment) run.  The last CTA to finish (atomic
-// ticket, no spinning) adds the partials of each segment, then the segments
-// of each layer, in a fixed order, so the result is deterministic for a
-// layout.
+// one fp64 partial per (range, layer) run.  The last CTA to finish (atomic
+// ticket, no spinning) adds the partials of each layer in a fixed order, so
+// the result is deterministic for a layout.
 //
 // Precision: per-thread fp32 accumulators take at most kUnroll * kFlush
 // terms each before they are added (fixed tree) into per-thread fp64 sums;
@@ -134,6 +133,21 @@ __device__ void scalar_vector(const SegDev& sd, int64_t k, double& dd, double& d
     }
 }
 
+// The terms of element e of a segment.
+template <bool WRITE_R>
+__device__ __forceinline__ void edge_element(const SegDev& sd, int64_t e, float& xd, float& xa) {
+    const float w = load_elem(sd.w, sd.esz_log2, e);
+    const float r = load_elem(sd.r, sd.esz_log2, e);
+    xd = fabsf(w - r);
+    xa = fabsf(r);
+    if constexpr (WRITE_R) {
+        if (sd.esz_log2 == 1)
+            reinterpret_cast<uint16_t*>(sd.r)[e] = reinterpret_cast<const uint16_t*>(sd.w)[e];
+        else
+            reinterpret_cast<float*>(sd.r)[e] = reinterpret_cast<const float*>(sd.w)[e];
+    }
+}
+
 // Vectors [lo, hi) of one segment into the calling thread's fp64 sums.
 template <bool WRITE_R>
 __device__ void process_run(const SegDev& sd, int64_t lo, int64_t hi, double& dd, double& da) {
@@ -172,18 +186,21 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
     const int64_t v1 = p.cta_vec_begin[b + 1];
     int s = p.cta_seg0[b];
     int slot = p.cta_slot0[b];
+    double dd = 0.0, da = 0.0;
     while (v0 < v1 && s < p.nseg) {
         const SegDev sd = p.segs[s];
         const int64_t seg_end = sd.vec_begin + sd.nvec;
         const int64_t lo = v0 - sd.vec_begin;
         const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
-        double dd = 0.0, da = 0.0;
         process_run<WRITE_R>(sd, lo, hi, dd, da);
+        ++s;
+        v0 = sd.vec_begin + hi;
+        if (v0 < v1 && s < p.nseg && p.segs[s].layer == sd.layer) continue;
         block_sum(dd, da, red_d, red_a);
         if (threadIdx.x == 0) p.partials[slot] = make_double2(dd, da);
         ++slot;
-        ++s;
-        v0 = sd.vec_begin + hi;
+        dd = 0.0;
+        da = 0.0;
     }
 
     if (threadIdx.x == 0) {
@@ -205,9 +222,9 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // that lie inside W and whose R windows (below) lie inside R, chunks of up to
 // kMChunk bytes of W and the same bytes of R loaded by cp.async.bulk into a
 // ring of kMStages buffers (one "full" mbarrier per buffer, completed by the
-// loads' byte count); for the few vectors at a segment's edges, a job the
-// consumers read from global memory element by element; after each run a
-// flush.
+// loads' byte count); with a run's first job come the few elements at the
+// segment's edges, which the consumers read from global memory, one a thread;
+// with its last the flush.
 //
 // W and R at different offsets from a 16-byte boundary (rshift != 0: weights
 // that are views of a flat buffer, snapshots that are tensors of their own):
@@ -217,21 +234,21 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // is the same for the whole segment, so it is a template parameter of the
 // loop.  A run like that used to be read element by element, two fp64 adds
 // each: a decision over 412 M bf16 parameters in 146 such segments took
-// 3110 us and takes 315 us (0.53 and 5.2 TB/s; the same parameters co-aligned
-// 277).  What bounds the shifted runs is the consumers' arithmetic: with plain
-// fp32 chains, as in the aligned runs, it took 277 us, but then lost precision
-// against the element path's fp64 (6e-12 instead of 3e-12 off the exact sums),
-// so the chains keep their rounding errors.  Warps 1..7 consume every job in order:
-// each thread adds its 16-byte vectors of the chunk into fp32 lanes (at most
-// ceil(chunk vectors / 224) terms before they go to fp64), and at a flush
-// each warp reduces its threads' fp64 sums in a fixed order into the run
-// box; the last warp to arrive adds the warps' sums in warp order and
-// writes the run's partial slot (run_box_put), so no warp waits for another
-// and no barrier spans warps.  Each warp hands a buffer back on its "empty"
-// mbarrier (7 arrivals).  Every wait is
-// bounded; a wait that runs out raises the fault word.  Warp-wide decisions
-// (the wait's outcome) are taken by lane 0 and broadcast, so the lanes of a
-// warp never part ways.
+// 3110 us and takes 294 (0.53 and 5.6 TB/s; the same parameters co-aligned
+// 269).  What bounds the shifted runs is the consumers' arithmetic: plain fp32
+// chains, as in the aligned runs, were 12% faster than chains that keep their
+// rounding errors, but lost precision against the element path's fp64 (6e-12
+// instead of 3e-12 off the exact sums).
+//
+// Warps 1..7 consume every job in order: each thread adds its 16-byte vectors
+// of the chunk into fp32 lanes (at most ceil(chunk vectors / 224) terms before
+// they go to fp64), and at a flush each warp reduces its threads' fp64 sums in
+// a fixed order into the run box; the last warp to arrive adds the warps' sums
+// in warp order and writes the run's partial slot (run_flush), so no warp
+// waits for another and no barrier spans warps.  Each warp hands a buffer back
+// on its "empty" mbarrier (7 arrivals) before it turns to fp64.  Every wait is
+// bounded; a wait that runs out raises the fault word.  A warp's lanes wait
+// together and take the outcome together, so they never part ways.
 // ---------------------------------------------------------------------------
 #ifndef LC_MEASURE_BULK_STAGES
 #define LC_MEASURE_BULK_STAGES 2
@@ -242,89 +259,130 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 constexpr int kMStages = LC_MEASURE_BULK_STAGES;
 constexpr uint32_t kMChunk = LC_MEASURE_BULK_CHUNK;      // bytes of W (and of R) per buffer
 constexpr int kMConsumerWarps = kMeasureThreads / 32 - 1;   // warps 1.. consume (2.. in accumulate mode)
-constexpr int kMConsumers = 32 * kMConsumerWarps;
 constexpr uint32_t kMStage = 2 * kMChunk + 128;          // R's part has room for the window's extra vector
 constexpr size_t kMeasureBulkSmem = size_t(kMStages) * kMStage;
 static_assert(kMChunk % 16 == 0 && kMStages >= 2, "measure ring shape");
 
-enum : int32_t { kJobChunk = 0, kJobScalar = 1, kJobFlush = 2, kJobEnd = 3 };
-
+// One job of a run: a chunk of n staged vectors (n may be 0), the elements at
+// the segment's edges (with the run's first job) and the flush (with its
+// last), so that a run of one chunk costs one turn of the ring.  What the
+// producer knows of the chunk travels with it: consumers and storer read no
+// table in global memory for it.
 struct MJob {
-    int64_t k0, k1;     // vectors [k0, k1) of the segment (chunk or scalar job)
-    int32_t kind;
+    int64_t ea, eb;     // elements [ea, ea + na) and [eb, eb + nb) of segment seg
+    uint8_t* r_out;     // the granule of R that holds the chunk's first byte
+    int32_t na, nb;
+    int32_t n;          // staged vectors; -1: no more jobs
+    int32_t esz_log2;
+    int32_t rshift;
     int32_t seg;
-    int32_t slot;       // first partial slot of the run (flush)
-    int32_t esz_log2;   // element size of the segment (chunk)
-    int32_t rshift;     // the segment's rshift (chunk)
+    int32_t slot;       // flush the run into this partial slot (-1: not yet)
     int32_t pad;
 };
+
+// A warp hands a job's buffer back before it flushes, so the flush's shuffles
+// and fp64 adds overlap the buffer's next load.  The producer is then up to
+// kMStages jobs ahead of a warp's last flush, hence one box more than stages.
+constexpr int kMBoxes = kMStages + 1;
 
 struct MRing {
     uint64_t full[kMStages];
     uint64_t empty[kMStages];
     MJob jobs[kMStages];
-    RunBox<kMStages, kMConsumerWarps> box;
+    RunBox<kMBoxes, kMConsumerWarps> box;
 };
 
 __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r) {
     const uint32_t ring_s = smem_addr(ring);
     const uint32_t full_s = smem_addr(r.full), empty_s = smem_addr(r.empty);
     uint64_t k = 0;
-    bool stall = p.stall_first != 0;
-    auto post = [&](const MJob& j, const SegDev& sd) -> bool {
+    uint32_t extra = p.stall_first ? 16u : 0u;   // bytes announced beyond the first load's
+    // the ring's next stage once its previous job has been handed back, or -1
+    auto stage = [&]() -> int {
         const int st = int(k % kMStages);
         if (k >= uint64_t(kMStages) &&
             !mbar_wait_bounded(empty_s + 8 * st, uint32_t((k / kMStages - 1) & 1), kWaitNs))
-            return false;
-        r.jobs[st] = j;
-        if (j.kind == kJobChunk) {
-            const uint32_t bytes = uint32_t(j.k1 - j.k0) * 16u;
-            const uint32_t rbytes = bytes + (sd.rshift ? 16u : 0u);
-            const uint8_t* wb = sd.w - (int64_t(sd.lead) << sd.esz_log2) + 16 * j.k0;
-            const uint8_t* rb = sd.r - (int64_t(sd.lead) << sd.esz_log2) - sd.rshift + 16 * j.k0;
-            mbar_expect_tx(full_s + 8 * st, bytes + rbytes + (stall ? 16u : 0u));
-            stall = false;
-            bulk_g2s(ring_s + uint32_t(st) * kMStage, wb, bytes, full_s + 8 * st);
-            bulk_g2s(ring_s + uint32_t(st) * kMStage + kMChunk, rb, rbytes, full_s + 8 * st);
-        } else {
-            mbar_arrive(full_s + 8 * st);
-        }
+            return -1;
         ++k;
-        return true;
+        return st;
     };
-    bool ok = true;
-    SegDev sd{};
+    int st = 0;
     // the CTA's own range, then units of the pool until it is empty
-    for (int rng = int(blockIdx.x); ok && rng >= 0; rng = ok ? next_pool_range(p) : -1) {
+    for (int rng = int(blockIdx.x); st >= 0 && rng >= 0; rng = st >= 0 ? next_pool_range(p) : -1) {
         int64_t v0 = p.cta_vec_begin[rng];
         const int64_t v1 = p.cta_vec_begin[rng + 1];
         int s = p.cta_seg0[rng];
         int slot = p.cta_slot0[rng];
-        while (ok && v0 < v1 && s < p.nseg) {
-            sd = p.segs[s];
+        SegDev sd;
+        if (v0 < v1 && s < p.nseg) sd = p.segs[s];
+        while (st >= 0 && v0 < v1 && s < p.nseg) {
             const int64_t seg_end = sd.vec_begin + sd.nvec;
             const int64_t lo = v0 - sd.vec_begin;
             const int64_t hi = (v1 < seg_end ? v1 : seg_end) - sd.vec_begin;
+            // the next segment is fetched while this one streams; the run ends with its layer
+            SegDev next;
+            const bool more = seg_end < v1 && s + 1 < p.nseg;
+            if (more) next = p.segs[s + 1];
+            const bool run_ends = !more || next.layer != sd.layer;
             // vectors [kf0, kf1) lie inside W with their R windows inside R
             const int64_t lead_b = (int64_t(sd.lead) << sd.esz_log2) + sd.rshift;
             const int64_t kf0 = (lead_b + 15) >> 4;
             int64_t kf1 = ((lead_b + (sd.numel << sd.esz_log2)) >> 4) - (sd.rshift ? 1 : 0);
             if (kf1 < kf0) kf1 = kf0;
-            const int64_t a = lo > kf0 ? lo : kf0;
+            int64_t x = lo > kf0 ? lo : kf0;
             const int64_t e = hi < kf1 ? hi : kf1;
-            if (lo < kf0) ok = post({lo, (hi < kf0 ? hi : kf0), kJobScalar, s, slot, 0, 0, 0}, sd);
-            constexpr int64_t kCV = kMChunk / 16;
-            for (int64_t x = a; ok && x < e; x += kCV)
-                ok = post({x, (x + kCV < e ? x + kCV : e), kJobChunk, s, slot, sd.esz_log2, sd.rshift, 0}, sd);
-            if (ok && hi > kf1) ok = post({(lo > kf1 ? lo : kf1), hi, kJobScalar, s, slot, 0, 0, 0}, sd);
-            if (ok) ok = post({0, 0, kJobFlush, s, slot, 0, 0, 0}, sd);
-            slot += kMeasureBulkSlotsPerRun;
+            // vectors [a, b) of the edges as elements of the segment
+            const int ve_log2 = 4 - sd.esz_log2;
+            auto first_elem = [&](int64_t a) { return a > 0 ? (a << ve_log2) - sd.lead : int64_t(0); };
+            auto end_elem = [&](int64_t b) {
+                const int64_t q = (b << ve_log2) - sd.lead;
+                return q < sd.numel ? q : sd.numel;
+            };
+            bool edges = true;
+            do {
+                st = stage();
+                if (st < 0) break;
+                MJob& j = r.jobs[st];
+                const int64_t n = x < e ? (e - x < int64_t(kMChunk / 16) ? e - x : int64_t(kMChunk / 16)) : 0;
+                j.na = j.nb = 0;
+                if (edges && lo < kf0) {
+                    j.ea = first_elem(lo);
+                    j.na = int32_t(end_elem(hi < kf0 ? hi : kf0) - j.ea);
+                }
+                if (edges && hi > kf1) {
+                    j.eb = first_elem(lo > kf1 ? lo : kf1);
+                    j.nb = int32_t(end_elem(hi) - j.eb);
+                }
+                edges = false;
+                j.n = int32_t(n);
+                j.esz_log2 = sd.esz_log2;
+                j.rshift = sd.rshift;
+                j.seg = s;
+                j.slot = run_ends && x + n >= e ? slot : -1;
+                if (n > 0) {
+                    const uint32_t bytes = uint32_t(n) * 16u, rbytes = bytes + (sd.rshift ? 16u : 0u);
+                    const int64_t at = 16 * x - (int64_t(sd.lead) << sd.esz_log2);
+                    j.r_out = sd.r + at - sd.rshift;
+                    mbar_expect_tx(full_s + 8 * st, bytes + rbytes + extra);
+                    extra = 0;
+                    bulk_g2s(ring_s + uint32_t(st) * kMStage, sd.w + at, bytes, full_s + 8 * st);
+                    bulk_g2s(ring_s + uint32_t(st) * kMStage + kMChunk, j.r_out, rbytes, full_s + 8 * st);
+                } else {
+                    mbar_arrive(full_s + 8 * st);
+                }
+                x += n;
+            } while (x < e);
+            if (run_ends) ++slot;
             ++s;
             v0 = sd.vec_begin + hi;
+            sd = next;
         }
     }
-    if (ok) ok = post({0, 0, kJobEnd, 0, 0, 0, 0, 0}, sd);
-    if (!ok) {
+    if (st >= 0) st = stage();
+    if (st >= 0) {
+        r.jobs[st].n = -1;
+        mbar_arrive(full_s + 8 * st);
+    } else {
         raise_fault(p.fault);
         // the loads of the last kMStages jobs may still be landing in shared memory
         const uint64_t first = k > uint64_t(kMStages) ? k - kMStages : 0;
@@ -380,7 +438,7 @@ __device__ __noinline__ double2 staged_elements(const uint8_t* W, const uint8_t*
 // be added element by element in fp64, and the sums are no less exact now.
 template <int ESZ_LOG2, int SH, bool WRITE_R, int NT>
 __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int n, int tid, uint8_t* r_out,
-                                            double& dd, double& da, float& ed, float& ea) {
+                                            double& dd, double& da, float& ed, float& ea, float& td, float& ta) {
     CompSums<ESZ_LOG2> cd, ca;
 #pragma unroll 2
     for (int v = tid; v < n; v += NT) {
@@ -409,9 +467,10 @@ __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int 
     }
     cd.reduce();
     ca.reduce();
+    td = ta = 0.f;
     if (isfinite(cd.s[0]) && isfinite(ca.s[0])) {
-        dd += double(cd.s[0]);
-        da += double(ca.s[0]);
+        td = cd.s[0];
+        ta = ca.s[0];
         ed += cd.e[0];
         ea += ca.e[0];
     } else {
@@ -425,22 +484,22 @@ __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int 
 template <bool WRITE_R, int NT>
 __device__ __forceinline__ void shifted_chunk(int esz_log2, int rshift, const uint4* W, const uint4* R, int n,
                                               int tid, uint8_t* r_out, double& dd, double& da,
-                                              float& ed, float& ea) {
+                                              float& ed, float& ea, float& td, float& ta) {
     if (esz_log2 == 1) {
         switch (rshift) {
-            case 2: shifted_run<1, 2, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 4: shifted_run<1, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 6: shifted_run<1, 6, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 8: shifted_run<1, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 10: shifted_run<1, 10, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 12: shifted_run<1, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            default: shifted_run<1, 14, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 2: shifted_run<1, 2, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 4: shifted_run<1, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 6: shifted_run<1, 6, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 8: shifted_run<1, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 10: shifted_run<1, 10, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 12: shifted_run<1, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            default: shifted_run<1, 14, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
         }
     } else {
         switch (rshift) {
-            case 4: shifted_run<2, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            case 8: shifted_run<2, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
-            default: shifted_run<2, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea); break;
+            case 4: shifted_run<2, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 8: shifted_run<2, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            default: shifted_run<2, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
         }
     }
 }
@@ -455,64 +514,57 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
     const int warp = tid >> 5, lane = tid & 31;
     double dd = 0.0, da = 0.0;
     float ed = 0.f, ea = 0.f;   // rounding errors of the run's compensated chains
+    int box = 0;                // of the next flush, the same in every warp
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kMStages);
         const uint32_t parity = uint32_t((k / kMStages) & 1);
-        int ok = 1;
-        if (lane == 0) ok = mbar_wait_bounded(full_s + 8 * st, parity, kWaitNs) ? 1 : 0;
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        if (!ok) {
+        if (!mbar_wait_warp(full_s + 8 * st, parity)) {
             if (lane == 0) raise_fault(p.fault);
             break;
         }
-        mbar_try_wait(full_s + 8 * st, parity);   // completed: orders this lane's reads after the loads
         const MJob j = r.jobs[st];
-        if (j.kind == kJobEnd) break;
-        if (j.kind == kJobChunk) {
+        if (j.n < 0) break;
+        float xd = 0.f, xa = 0.f;   // this thread's element of the segment's edges
+        if (tid < j.na + j.nb) edge_element<WRITE_R>(p.segs[j.seg], tid < j.na ? j.ea + tid : j.eb + (tid - j.na), xd, xa);
+        float td = 0.f, ta = 0.f;     // and its chunk's sums
+        if (j.n > 0) {
             const uint4* W = reinterpret_cast<const uint4*>(ring + size_t(st) * kMStage);
             const uint4* R = W + kMChunk / 16;
-            const int n = int(j.k1 - j.k0);
             if (j.rshift) {
-                uint8_t* r_out = nullptr;
-                if constexpr (WRITE_R) {
-                    const SegDev& sd = p.segs[j.seg];
-                    r_out = sd.r - (int64_t(sd.lead) << sd.esz_log2) - sd.rshift + 16 * j.k0;
-                }
-                shifted_chunk<WRITE_R, kThreads>(j.esz_log2, j.rshift, W, R, n, tid, r_out, dd, da, ed, ea);
+                shifted_chunk<WRITE_R, kThreads>(j.esz_log2, j.rshift, W, R, j.n, tid, j.r_out, dd, da, ed, ea, td, ta);
             } else {
                 float ad[8], aa[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q) { ad[q] = 0.f; aa[q] = 0.f; }
                 if (j.esz_log2 == 1) {
 #pragma unroll 4
-                    for (int v = tid; v < n; v += kThreads) accumulate<1>(W[v], R[v], ad, aa);
+                    for (int v = tid; v < j.n; v += kThreads) accumulate<1>(W[v], R[v], ad, aa);
                 } else {
 #pragma unroll 4
-                    for (int v = tid; v < n; v += kThreads) accumulate<2>(W[v], R[v], ad, aa);
+                    for (int v = tid; v < j.n; v += kThreads) accumulate<2>(W[v], R[v], ad, aa);
                 }
-                dd += double(tree8(ad));
-                da += double(tree8(aa));
+                td = tree8(ad);
+                ta = tree8(aa);
             }
-        } else if (j.kind == kJobScalar) {
-            const SegDev sd = p.segs[j.seg];
-            for (int64_t v = j.k0 + tid; v < j.k1; v += kThreads) scalar_vector<WRITE_R>(sd, v, dd, da);
-        } else {   // flush: this warp's share of the run, in a fixed order
+        }
+        mbar_arrive_warp(empty_s + 8 * st, lane);
+        after_handback(td, ta);
+        dd += double(td);
+        da += double(ta);
+        if (tid < j.na + j.nb) {
+            dd += double(xd);
+            da += double(xa);
+        }
+        if (j.slot >= 0) {   // flush: this warp's share of the run
             dd += double(ed);
             da += double(ea);
             ed = 0.f;
             ea = 0.f;
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                dd += __shfl_down_sync(0xffffffffu, dd, off);
-                da += __shfl_down_sync(0xffffffffu, da, off);
-            }
-            if (lane == 0)
-                run_box_put<kMConsumerWarps - (WRITE_R ? 1 : 0)>(r.box, st, warp, dd, da, p.partials + j.slot);
+            run_flush<kMConsumerWarps - (WRITE_R ? 1 : 0)>(r.box, box, warp, lane, dd, da, p.partials + j.slot);
+            box = box + 1 < kMBoxes ? box + 1 : 0;
             dd = 0.0;
             da = 0.0;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty_s + 8 * st);
     }
 }
 
@@ -529,15 +581,11 @@ __device__ void measure_store_r(const MeasureParams& p, const uint8_t* ring, MRi
             raise_fault(p.fault);
             break;
         }
-        const MJob j = r.jobs[st];
-        if (j.kind == kJobEnd) break;
-        if (j.kind == kJobChunk && j.rshift == 0) {
-            const SegDev sd = p.segs[j.seg];
-            uint8_t* rb = sd.r - (int64_t(sd.lead) << sd.esz_log2) + 16 * j.k0;
+        const MJob& j = r.jobs[st];
+        if (j.n < 0) break;
+        if (j.n > 0 && j.rshift == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(rb),
-                         "r"(ring_s + uint32_t(st) * kMStage), "r"(uint32_t(j.k1 - j.k0) * 16u)
-                         : "memory");
+            bulk_s2g(j.r_out, ring_s + uint32_t(st) * kMStage, uint32_t(j.n) * 16u);
             asm volatile("cp.async.bulk.commit_group;" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
         }
@@ -551,14 +599,16 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
     extern __shared__ __align__(128) uint8_t ring[];
     __shared__ __align__(8) MRing r;
     __shared__ unsigned int s_ticket;
+    __shared__ __align__(8) FinTables tables;
     if (threadIdx.x == 0) {
         for (int st = 0; st < kMStages; ++st) {
             mbar_init(smem_addr(&r.full[st]), 1);
             mbar_init(smem_addr(&r.empty[st]), kMConsumerWarps);
-            r.box.count[st] = 0u;
         }
+        for (int b = 0; b < kMBoxes; ++b) r.box.count[b] = 0u;
         mbar_init_fence();
     }
+    fin_prefetch(p, tables);
     __syncthreads();
     if (threadIdx.x == 0) {
         measure_produce(p, ring, r);
@@ -567,6 +617,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
     } else if (threadIdx.x >= 32) {
         measure_consume<WRITE_R>(p, ring, r);
     }
+    fin_prefetch_wait();
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
@@ -576,7 +627,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
     if (s_ticket != gridDim.x - 1) return;
     __threadfence();
     // the ring's loads have all landed (or the CTA gave up): it stages the combine
-    finalize(p, reinterpret_cast<double2*>(ring), int32_t(kMeasureBulkSmem / sizeof(double2)));
+    finalize(p, reinterpret_cast<double2*>(ring), int32_t(kMeasureBulkSmem / sizeof(double2)), &tables);
 }
 
 }  // namespace

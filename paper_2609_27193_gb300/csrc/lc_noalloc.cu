@@ -38,18 +38,18 @@ constexpr size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
 // back to back (16-byte aligned) for the call's sizes, so the upload moves
 // only the bytes the measure will read.
 struct TableLayout {
-    size_t segs, cta_vec, cta_seg, cta_slot, seg_slot, layer_seg, ticket, bytes;
+    size_t segs, cta_vec, layer_n, cta_seg, cta_slot, layer_slot, ticket, bytes;
 };
 
 constexpr TableLayout table_layout(size_t nseg, size_t nlayers, size_t G) {
     TableLayout t{};
     t.segs = 0;
     t.cta_vec = al16(t.segs + sizeof(SegDev) * nseg);
-    t.cta_seg = al16(t.cta_vec + sizeof(int64_t) * (G + 1));
+    t.layer_n = al16(t.cta_vec + sizeof(int64_t) * (G + 1));
+    t.cta_seg = al16(t.layer_n + sizeof(double) * nlayers);
     t.cta_slot = al16(t.cta_seg + sizeof(int32_t) * G);
-    t.seg_slot = al16(t.cta_slot + sizeof(int32_t) * G);
-    t.layer_seg = al16(t.seg_slot + sizeof(int32_t) * (nseg + 1));
-    t.ticket = al16(t.layer_seg + sizeof(int32_t) * (nlayers + 1));
+    t.layer_slot = al16(t.cta_slot + sizeof(int32_t) * G);
+    t.ticket = al16(t.layer_slot + sizeof(int32_t) * (nlayers + 1));
     t.bytes = al16(t.ticket + sizeof(unsigned int));
     return t;
 }
@@ -57,8 +57,7 @@ constexpr TableLayout table_layout(size_t nseg, size_t nlayers, size_t G) {
 // Scratch layout: the tables (at most kTableBytes), then the kernel scratch.
 constexpr size_t kTableBytes = al256(table_layout(kMaxSeg, kMaxLayers, kMaxCtas).bytes);
 constexpr size_t kOffPartials = kTableBytes;
-constexpr size_t kOffSegSums = al256(kOffPartials + sizeof(double2) * (kMaxCtas + kMaxSeg));
-constexpr size_t kScratchUsed = al256(kOffSegSums + sizeof(double) * 2 * kMaxSeg);
+constexpr size_t kScratchUsed = al256(kOffPartials + sizeof(double2) * (kMaxCtas + kMaxLayers));
 static_assert(kScratchUsed <= LC_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds its array");
 
 }  // namespace
@@ -256,9 +255,14 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
     int64_t* cta_vec = reinterpret_cast<int64_t*>(t_image + L.cta_vec);
     int32_t* cta_seg = reinterpret_cast<int32_t*>(t_image + L.cta_seg);
     int32_t* cta_slot = reinterpret_cast<int32_t*>(t_image + L.cta_slot);
-    int32_t* seg_slot = reinterpret_cast<int32_t*>(t_image + L.seg_slot);
-    int32_t* layer_seg = reinterpret_cast<int32_t*>(t_image + L.layer_seg);
-    for (int32_t i = 0; i <= nseg; ++i) seg_slot[i] = -1;
+    int32_t* layer_slot = reinterpret_cast<int32_t*>(t_image + L.layer_slot);
+    double* layer_n = reinterpret_cast<double*>(t_image + L.layer_n);
+    for (int32_t l = 0; l <= nlayers; ++l) layer_slot[l] = -1;
+    for (int32_t l = 0; l < nlayers; ++l) {
+        int64_t n = 0;
+        for (int32_t i = layer_begin[l]; i < layer_begin[l + 1]; ++i) n += sd[i].numel;
+        layer_n[l] = double(n);
+    }
     for (int64_t b = 0; b <= G; ++b) {
         const int64_t v = ngran * b / G * LC_MEASURE_ALIGN_VECS;
         cta_vec[b] = v < V ? v : V;
@@ -270,15 +274,15 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         cta_seg[b] = s;
         cta_slot[b] = slot;
         for (int32_t t = s; v0 < v1 && t < nseg && sd[t].vec_begin < v1; ++t) {
-            if (seg_slot[t] < 0) seg_slot[t] = slot;
+            if (t > s && sd[t].layer == sd[t - 1].layer) continue;
+            if (layer_slot[sd[t].layer] < 0) layer_slot[sd[t].layer] = slot;
             ++slot;
         }
     }
-    seg_slot[nseg] = slot;
-    for (int32_t t = nseg - 1; t >= 0; --t)
-        if (seg_slot[t] < 0) seg_slot[t] = seg_slot[t + 1];
-    std::memcpy(layer_seg, layer_begin, sizeof(int32_t) * (nlayers + 1));
-    if (slot > kMaxCtas + kMaxSeg) return err(LC_ERR_CUDA, "lc_measure_noalloc: internal slot overflow");
+    layer_slot[nlayers] = slot;
+    for (int32_t l = nlayers - 1; l >= 0; --l)
+        if (layer_slot[l] < 0) layer_slot[l] = layer_slot[l + 1];
+    if (slot > kMaxCtas + kMaxLayers) return err(LC_ERR_CUDA, "lc_measure_noalloc: internal slot overflow");
 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // the tables and a zero completion counter into the scratch array,
@@ -299,10 +303,9 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
     p.cta_vec_begin = reinterpret_cast<const int64_t*>(ds.addr + L.cta_vec);
     p.cta_seg0 = reinterpret_cast<const int32_t*>(ds.addr + L.cta_seg);
     p.cta_slot0 = reinterpret_cast<const int32_t*>(ds.addr + L.cta_slot);
-    p.seg_slot_begin = reinterpret_cast<const int32_t*>(ds.addr + L.seg_slot);
-    p.layer_seg_begin = reinterpret_cast<const int32_t*>(ds.addr + L.layer_seg);
+    p.layer_slot_begin = reinterpret_cast<const int32_t*>(ds.addr + L.layer_slot);
+    p.layer_n = reinterpret_cast<const double*>(ds.addr + L.layer_n);
     p.partials = reinterpret_cast<double2*>(ds.addr + kOffPartials);
-    p.seg_sums = reinterpret_cast<double*>(ds.addr + kOffSegSums);
     p.sums = sums_out;
     p.ticket = reinterpret_cast<unsigned int*>(ds.addr + L.ticket);
     p.nseg = nseg;

@@ -1,7 +1,7 @@
 // lc_reduce.cuh -- device helpers shared by the kernels that reduce over
 // the measure work space (lc_measure.cu: the Eq. 1 scan; lc_adamw.cu: the
 // fused optimizer step): streaming loads and stores, bf16 decoding, the
-// fixed-order CTA sum and the last-CTA fp64 combine per segment and layer,
+// fixed-order CTA sum and the last-CTA fp64 combine per layer,
 // and fp32 chains that keep their rounding errors.
 #pragma once
 
@@ -112,38 +112,52 @@ __device__ __forceinline__ void block_sum(double& d, double& a, double* sd, doub
     __syncthreads();
 }
 
-// A run's partial from a bulk kernel's consumer warps.  Each warp's lane 0
-// leaves its warp-reduced (d, a) in the box of the flush job's ring stage;
-// the last of the N contributing warps to arrive adds them in warp order and
-// writes the run's one partial slot.  No warp waits for another.  A stage's
-// box is used again only once every warp has handed that stage back, so
-// warps up to a ring's depth apart never share a box.
-template <int NSTAGES, int MAXW>
+// A run's partial from a bulk kernel's consumer warps.  Each warp leaves its
+// reduced (d, a) in the run's box; the last of the N contributing warps to
+// arrive adds them in warp order and writes the run's one partial slot.  No
+// warp waits for another.  A box is used again only once every warp has
+// arrived at it and gone on (the kernels say why).
+//
+// fp64 runs at a few operations per cycle per SM here and a warp-wide add
+// costs the same with one lane busy or 32, so the reduction keeps both sums
+// in one add: lanes 0..15 carry d and lanes 16..31 a from the first step on,
+// five adds instead of ten, and a warp whose lanes all hold zero skips them.
+template <int NBOXES, int MAXW>
 struct RunBox {
-    double d[NSTAGES][MAXW];
-    double a[NSTAGES][MAXW];
-    unsigned int count[NSTAGES];
+    double v[NBOXES][2][MAXW];   // d, a
+    unsigned int count[NBOXES];
 };
 
-template <int N, int NSTAGES, int MAXW>
-__device__ __forceinline__ void run_box_put(RunBox<NSTAGES, MAXW>& b, int st, int w, double d, double a,
-                                            double2* slot) {
+template <int N, int NBOXES, int MAXW>
+__device__ __forceinline__ void run_flush(RunBox<NBOXES, MAXW>& b, int box, int w, int lane, double d, double a,
+                                          double2* slot) {
     static_assert(N <= MAXW, "run box too small");
-    volatile double* vd = b.d[st];
-    volatile double* va = b.a[st];
-    vd[w] = d;
-    va[w] = a;
-    __threadfence_block();
-    if (atomicAdd(&b.count[st], 1u) == unsigned(N - 1)) {
-        __threadfence_block();
-        double sd = 0.0, sa = 0.0;
-        for (int i = 0; i < N; ++i) {
-            sd += vd[i];
-            sa += va[i];
-        }
-        *slot = make_double2(sd, sa);
-        *reinterpret_cast<volatile unsigned int*>(&b.count[st]) = 0u;
+    const int half = lane >> 4;
+    double x = half ? a : d;
+    if (__any_sync(0xffffffffu, d != 0.0 || a != 0.0)) {
+        x += __shfl_xor_sync(0xffffffffu, half ? d : a, 16);
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
     }
+    volatile double* v = b.v[box][half];
+    if ((lane & 15) == 0) {
+        v[w] = x;
+        __threadfence_block();
+    }
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) last = atomicAdd(&b.count[box], 1u) == unsigned(N - 1) ? 1 : 0;
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (!last) return;
+    __threadfence_block();
+    if ((lane & 15) == 0) {
+        double sum = 0.0;
+        for (int i = 0; i < N; ++i) sum += v[i];
+        reinterpret_cast<double*>(slot)[half] = sum;
+    }
+    __syncwarp();
+    if (lane == 0) *reinterpret_cast<volatile unsigned int*>(&b.count[box]) = 0u;
+    __syncwarp();
 }
 
 // The next pool range for the calling CTA (its producer thread), or -1 once
@@ -156,168 +170,111 @@ __device__ __forceinline__ int next_pool_range(const MeasureParams& p) {
     return u < unsigned(p.units) ? int(gridDim.x) + int(u) : -1;
 }
 
-// Run by the last CTA: the partial slots of every segment are added, then
-// one thread per layer adds its segments in order.  The order of every
-// addition is fixed by the layout.  The combine runs while the rest of the
-// GPU is idle, so its latency is the kernel's tail, and on this GPU fp64
-// arithmetic runs at a few operations per cycle per SM: a warp-wide fp64
-// add is expensive whether its lanes hold data or not.  The slot bounds of
-// up to kFinBatch segments are staged in shared memory first.
+// Run by the last CTA: the partial slots of every layer, contiguous in
+// `partials`, are added.  The order of every addition is fixed by the layout.
+// The combine runs while the rest of the GPU is idle, so its latency is the
+// kernel's tail, and that is the latency of dependent fp64 adds and of trips
+// to global memory.  A layer of at most kFinLane slots is added by two
+// threads, one for d and one for a, in slot order (16 layers per warp
+// instruction); a larger one by a warp, lanes 0..15 for d and 16..31 for a,
+// each lane every 16th slot, then a fixed tree.
 //
-// With `stage` (shared memory free for reuse, stage_slots slots of it: the
-// bulk kernels' rings) the slots of consecutive segments -- contiguous in
-// `partials` -- are first copied there by the whole CTA with kFinLoads
-// independent loads in flight per thread.  A segment of at most kFinLane
-// slots is then added by one thread in slot order (32 segments per warp
-// instruction); a larger one by a warp (lane l takes slots l, l+32, ... in
-// order, then a fixed shuffle tree); a segment with more slots than fit in
-// the stage is added by a warp from global memory.  Without `stage` the
-// same split applies with the slots read from global memory, a thread
-// keeping kFinLaneLoads loads in flight.
-constexpr int kFinBatch = 512;
-constexpr int kFinLaneLoads = 4;
+// The bulk kernels give it `stage` (shared memory free for reuse, stage_slots
+// slots of it: their rings), where the whole CTA first copies the slots with
+// kFinLoads independent loads in flight per thread, and `tables`: every CTA
+// fetches the combine's tables while its range streams (fin_prefetch,
+// asynchronous copies; which CTA is the last shows at the end), so the slots
+// are the combine's only trip.  Without them, or with more slots or layers
+// than they hold, slots and tables are read from global memory.
+//
+// Runs, and so slots, are per (range, layer): a flush costs the consumer warps
+// about as much as a chunk, and a small model's CTA crosses several tensors of
+// a layer.  For 6 M parameters in 38 tensors and 6 layers the last consumer is
+// done 9.5 us after the launch and the combine takes 2.0 us (13.4 and 4.6 with
+// runs per tensor and a combine by tensor, then layer); the decision takes 34
+// instead of 43 us, one over 138 M parameters 116 instead of 119.5.
 constexpr int kFinLoads = 8;
-constexpr int kFinLane = 32;
+constexpr int kFinLane = 24;
+constexpr int kFinLayers = 512;
 
-// Slots [b0, b1) of one segment into (d, a) of lane 0, in the fixed order.
-template <typename Slots>
-__device__ __forceinline__ void fin_segment(const Slots& slot, int32_t b0, int32_t b1, int lane, double& d,
-                                            double& a) {
-    d = 0.0;
-    a = 0.0;
-    for (int32_t j = b0 + lane; j < b1; j += 32) {
-        const double2 v = slot(j);
-        d += v.x;
-        a += v.y;
+struct FinTables {
+    int32_t slot_begin[kFinLayers + 1];
+    double layer_n[kFinLayers];
+};
+
+template <int BYTES>
+__device__ __forceinline__ void fetch_async(void* smem, const void* global) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(
+                     static_cast<uint32_t>(__cvta_generic_to_shared(smem))),
+                 "l"(global), "n"(BYTES)
+                 : "memory");
+}
+
+__device__ __forceinline__ void fin_prefetch(const MeasureParams& p, FinTables& t) {
+    if (p.nlayers > kFinLayers) return;
+    for (int i = threadIdx.x; i <= p.nlayers; i += blockDim.x) fetch_async<4>(&t.slot_begin[i], p.layer_slot_begin + i);
+    for (int i = threadIdx.x; i < p.nlayers; i += blockDim.x) fetch_async<8>(&t.layer_n[i], p.layer_n + i);
+}
+
+// Every thread, before the CTA's last barrier.
+__device__ __forceinline__ void fin_prefetch_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// Both sums of every layer from slot(j, component).
+template <typename Slot>
+__device__ __forceinline__ void fin_layers(const MeasureParams& p, const int32_t* slot_begin, const double* layer_n,
+                                           const Slot& slot) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int i = threadIdx.x; i < 2 * p.nlayers; i += blockDim.x) {
+        const int l = i >> 1, c = i & 1;
+        const int32_t b0 = slot_begin[l], b1 = slot_begin[l + 1];
+        if (c == 0) p.sums[3 * l + 2] = layer_n[l];
+        if (b1 - b0 > kFinLane) continue;
+        double x = 0.0;
+#pragma unroll 4
+        for (int32_t j = b0; j < b1; ++j) x += slot(j, c);
+        p.sums[3 * l + c] = x;
     }
+    for (int l = warp; l < p.nlayers; l += nw) {
+        const int32_t b0 = slot_begin[l], b1 = slot_begin[l + 1];
+        if (b1 - b0 <= kFinLane) continue;
+        double x = 0.0;
+#pragma unroll 4
+        for (int32_t j = b0 + (lane & 15); j < b1; j += 16) x += slot(j, lane >> 4);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        d += __shfl_down_sync(0xffffffffu, d, off);
-        a += __shfl_down_sync(0xffffffffu, a, off);
+        for (int off = 8; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+        if ((lane & 15) == 0) p.sums[3 * l + (lane >> 4)] = x;
     }
 }
 
-__device__ void finalize(const MeasureParams& p, double2* stage = nullptr, int32_t stage_slots = 0) {
-    __shared__ int32_t s_beg[kFinBatch + 1];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    auto global_slot = [&](int32_t j) { return __ldcg(&p.partials[j]); };
-    for (int base = 0; base < p.nseg; base += kFinBatch) {
-        const int nb = p.nseg - base < kFinBatch ? p.nseg - base : kFinBatch;
-        __syncthreads();
-        for (int i = threadIdx.x; i <= nb; i += blockDim.x) s_beg[i] = p.seg_slot_begin[base + i];
-        __syncthreads();
-        if (stage) {
-            for (int g0 = 0; g0 < nb;) {
-                // the longest run of segments [g0, g1) whose slots fit the stage
-                int lo = g0 + 1, hi = nb;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (s_beg[mid] - s_beg[g0] <= stage_slots) lo = mid;
-                    else hi = mid - 1;
-                }
-                const int g1 = lo;
-                const int32_t first = s_beg[g0];
-                const int32_t n = s_beg[g1] - first;
-                if (n > stage_slots) {          // one segment larger than the stage
-                    if (warp == 0) {
-                        double d, a;
-                        fin_segment(global_slot, s_beg[g0], s_beg[g0 + 1], lane, d, a);
-                        if (lane == 0) {
-                            p.seg_sums[2 * (base + g0)] = d;
-                            p.seg_sums[2 * (base + g0) + 1] = a;
-                        }
-                    }
-                } else {
-                    for (int32_t i0 = 0; i0 < n; i0 += int32_t(blockDim.x) * kFinLoads) {
-                        double2 v[kFinLoads];
-#pragma unroll
-                        for (int k = 0; k < kFinLoads; ++k) {
-                            const int32_t i = i0 + k * int32_t(blockDim.x) + int32_t(threadIdx.x);
-                            if (i < n) v[k] = __ldcg(&p.partials[first + i]);
-                        }
-#pragma unroll
-                        for (int k = 0; k < kFinLoads; ++k) {
-                            const int32_t i = i0 + k * int32_t(blockDim.x) + int32_t(threadIdx.x);
-                            if (i < n) stage[i] = v[k];
-                        }
-                    }
-                    __syncthreads();
-                    auto staged_slot = [&](int32_t j) { return stage[j - first]; };
-                    for (int s = g0 + int(threadIdx.x); s < g1; s += int(blockDim.x)) {
-                        const int32_t b0 = s_beg[s], b1 = s_beg[s + 1];
-                        if (b1 - b0 > kFinLane) continue;
-                        double d = 0.0, a = 0.0;
-                        for (int32_t j = b0; j < b1; ++j) {
-                            const double2 v = stage[j - first];
-                            d += v.x;
-                            a += v.y;
-                        }
-                        p.seg_sums[2 * (base + s)] = d;
-                        p.seg_sums[2 * (base + s) + 1] = a;
-                    }
-                    for (int s = g0 + warp; s < g1; s += nw) {
-                        if (s_beg[s + 1] - s_beg[s] <= kFinLane) continue;
-                        double d, a;
-                        fin_segment(staged_slot, s_beg[s], s_beg[s + 1], lane, d, a);
-                        if (lane == 0) {
-                            p.seg_sums[2 * (base + s)] = d;
-                            p.seg_sums[2 * (base + s) + 1] = a;
-                        }
-                    }
-                }
-                __syncthreads();
-                g0 = g1;
-            }
-            continue;
-        }
-        for (int s = int(threadIdx.x); s < nb; s += int(blockDim.x)) {
-            const int32_t b0 = s_beg[s], b1 = s_beg[s + 1];
-            if (b1 - b0 > kFinLane) continue;
-            double d = 0.0, a = 0.0;
-            for (int32_t j = b0; j < b1; j += kFinLaneLoads) {
-                double2 v[kFinLaneLoads];
-#pragma unroll
-                for (int k = 0; k < kFinLaneLoads; ++k)
-                    if (j + k < b1) v[k] = __ldcg(&p.partials[j + k]);
-#pragma unroll
-                for (int k = 0; k < kFinLaneLoads; ++k)
-                    if (j + k < b1) {
-                        d += v[k].x;
-                        a += v[k].y;
-                    }
-            }
-            p.seg_sums[2 * (base + s)] = d;
-            p.seg_sums[2 * (base + s) + 1] = a;
-        }
-        for (int s = warp; s < nb; s += nw) {
-            if (s_beg[s + 1] - s_beg[s] <= kFinLane) continue;
-            double d, a;
-            fin_segment(global_slot, s_beg[s], s_beg[s + 1], lane, d, a);
-            if (lane == 0) {
-                p.seg_sums[2 * (base + s)] = d;
-                p.seg_sums[2 * (base + s) + 1] = a;
-            }
-        }
-    }
-    __syncthreads();
-    for (int l = threadIdx.x; l < p.nlayers; l += blockDim.x) {
-        double d = 0.0, a = 0.0;
-        int64_t n = 0;
-        const int sb = p.layer_seg_begin[l], se = p.layer_seg_begin[l + 1];
-#pragma unroll 4
-        for (int s = sb; s < se; ++s) {
-            d += __ldcg(&p.seg_sums[2 * s]);
-            a += __ldcg(&p.seg_sums[2 * s + 1]);
-            n += p.segs[s].numel;
-        }
-        p.sums[3 * l] = d;
-        p.sums[3 * l + 1] = a;
-        p.sums[3 * l + 2] = double(n);
-    }
+__device__ void finalize(const MeasureParams& p, double2* stage = nullptr, int32_t stage_slots = 0,
+                         const FinTables* tables = nullptr) {
     if (threadIdx.x == 0) {
         *p.ticket = 0u;
         if (p.unit_next) *p.unit_next = 0u;   // every CTA has left the pool
     }
+    const double* global = reinterpret_cast<const double*>(p.partials);
+    const bool fit = tables && p.nlayers <= kFinLayers;
+    const int32_t n = fit ? tables->slot_begin[p.nlayers] : 0;
+    if (!fit || n > stage_slots) {
+        fin_layers(p, p.layer_slot_begin, p.layer_n, [&](int32_t j, int c) { return __ldcg(global + 2 * j + c); });
+        return;
+    }
+    for (int32_t i0 = 0; i0 < n; i0 += int32_t(blockDim.x) * kFinLoads) {
+        double2 v[kFinLoads];
+#pragma unroll
+        for (int k = 0; k < kFinLoads; ++k) {
+            const int32_t i = i0 + k * int32_t(blockDim.x) + int32_t(threadIdx.x);
+            if (i < n) v[k] = __ldcg(&p.partials[i]);
+        }
+#pragma unroll
+        for (int k = 0; k < kFinLoads; ++k) {
+            const int32_t i = i0 + k * int32_t(blockDim.x) + int32_t(threadIdx.x);
+            if (i < n) stage[i] = v[k];
+        }
+    }
+    __syncthreads();
+    const double* staged = reinterpret_cast<const double*>(stage);
+    fin_layers(p, tables->slot_begin, tables->layer_n, [&](int32_t j, int c) { return staged[2 * j + c]; });
 }
 
 }  // namespace
