@@ -394,9 +394,9 @@ struct lc_ctx {
     CopyDesc* d_commit_desc = nullptr;
     CopyDesc* d_restore_desc = nullptr;
     uint8_t* d_result = nullptr;
-    uint8_t* h_result = nullptr;           // pinned
+    uint8_t* h_result = nullptr;           // pinned, written by the select kernel
+    uint8_t* d_h_result = nullptr;         // its device address
     ResultLayout rl{};
-    cudaEvent_t ev_result = nullptr;
 
     // staging ring
     uint8_t* d_staging = nullptr;
@@ -415,7 +415,8 @@ struct lc_ctx {
 
     // device-driven steps: pinned decision blocks of steps still in flight
     struct AsyncSlot {
-        uint8_t* host = nullptr;   // pinned copy of the decision block
+        uint8_t* host = nullptr;   // pinned decision block
+        uint8_t* host_dev = nullptr;   // its device address
         cudaEvent_t done = nullptr;
         int64_t step = -1;
         bool busy = false;
@@ -459,6 +460,37 @@ lc_status check_copy_fault(const lc_ctx* ctx, const char* what) {
     if (ctx->h_fault && *reinterpret_cast<volatile const uint32_t*>(ctx->h_fault))
         return fail(LC_ERR_TIMEOUT, "%s: a bulk-engine copy gave up waiting for its loads", what);
     return LC_OK;
+}
+
+lc_status alloc_host_block(lc_ctx* ctx, uint8_t** host, uint8_t** dev) {
+    LC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(host), ctx->rl.total, cudaHostAllocMapped));
+    std::memset(*host, 0, ctx->rl.total);
+    LC_CUDA(cudaHostGetDevicePointer(reinterpret_cast<void**>(dev), *host, 0));
+    return LC_OK;
+}
+
+// Polls the decision block's magic word, which the select kernel writes last,
+// until it is there or the configured timeout passes.  The stream is asked
+// now and then: an error on it would leave the word unwritten.
+lc_status wait_decision(lc_ctx* ctx, const uint32_t* magic, const char* what) {
+    using clk = std::chrono::steady_clock;
+    const auto t0 = clk::now();
+    for (long spins = 1;; ++spins) {
+        if (__atomic_load_n(magic, __ATOMIC_ACQUIRE) == kResultMagic) return LC_OK;
+        if (spins % 256) continue;
+        const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(clk::now() - t0).count();
+        if (ms > ctx->cfg.timeout_ms)
+            return fail(LC_ERR_TIMEOUT, "%s: not complete after %d ms", what, ctx->cfg.timeout_ms);
+        if (ms < 2) continue;
+        const cudaError_t q = cudaStreamQuery(ctx->stream);
+        if (q != cudaSuccess && q != cudaErrorNotReady) {
+            cudaGetLastError();
+            return fail(LC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(q));
+        }
+        if (q == cudaSuccess && __atomic_load_n(magic, __ATOMIC_ACQUIRE) != kResultMagic)
+            return fail(LC_ERR_CUDA, "%s: the decision was not written", what);
+        if (ms > 20) std::this_thread::sleep_for(std::chrono::microseconds(50));
+    }
 }
 
 // Engine and grid of a copy launch whose stream-side buffer is `base`
@@ -594,7 +626,6 @@ extern "C" lc_status lc_create(lc_ctx** out, int device, void* cuda_stream, cons
     ctx->cfg = c;
     ctx->sms = prop.multiProcessorCount;
     cudaError_t e = cudaStreamCreateWithFlags(&ctx->copy_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_result, cudaEventDisableTiming);
     for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
         e = cudaEventCreateWithFlags(&ctx->ev_slot_free[i], cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ctx->ev_slot_filled[i], cudaEventDisableTiming);
@@ -649,7 +680,6 @@ extern "C" void lc_destroy(lc_ctx* ctx) {
     cudaFree(ctx->d_staging);
     if (ctx->h_result) cudaFreeHost(ctx->h_result);
     if (ctx->h_fault) cudaFreeHost(ctx->h_fault);
-    if (ctx->ev_result) cudaEventDestroy(ctx->ev_result);
     for (int i = 0; i < 2; ++i) {
         if (ctx->ev_slot_free[i]) cudaEventDestroy(ctx->ev_slot_free[i]);
         if (ctx->ev_slot_filled[i]) cudaEventDestroy(ctx->ev_slot_filled[i]);
@@ -936,12 +966,12 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     const size_t o_lwsec = tp.take(sizeof(int32_t) * nlayers);
     const size_t o_lcw = tp.take(sizeof(uint64_t) * nlayers);
     const size_t o_secs = tp.take(sizeof(SectionDev) * std::max(1, nsec));
-    const size_t o_scratch = tp.take(sizeof(int64_t) * 3 * nlayers);
+    const size_t o_place = tp.take(sizeof(LayerPlace) * nlayers);
     const size_t o_accsave = tp.take(sizeof(double) * nlayers);
     const size_t o_tlsave = tp.take(sizeof(int64_t) * nlayers);
     const size_t o_stepctr = tp.take(sizeof(int64_t));
     ctx->rl = result_layout(nlayers);
-    const size_t o_result = tp.take(ctx->rl.total);
+    const size_t o_result = tp.take(sizeof(ResultHeader));
     const size_t o_pdesc = tp.take(sizeof(CopyDesc) * std::max(1, nsec));
     const size_t o_cdesc = tp.take(sizeof(CopyDesc) * nseg);
     const size_t o_rdesc = tp.take(sizeof(CopyDesc) * std::max(1, nsec));
@@ -1018,7 +1048,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     sp.layer_wsec_count = reinterpret_cast<const int32_t*>(base + o_lwsec);
     sp.layer_commit_work = reinterpret_cast<const uint64_t*>(base + o_lcw);
     sp.secs = reinterpret_cast<const SectionDev*>(base + o_secs);
-    sp.layer_scratch = reinterpret_cast<int64_t*>(base + o_scratch);
+    sp.layer_place = reinterpret_cast<LayerPlace*>(base + o_place);
     sp.acc_save = reinterpret_cast<double*>(base + o_accsave);
     sp.tl_save = reinterpret_cast<int64_t*>(base + o_tlsave);
     sp.step_counter = reinterpret_cast<int64_t*>(base + o_stepctr);
@@ -1028,6 +1058,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     sp.pack_desc = reinterpret_cast<CopyDesc*>(base + o_pdesc);
     sp.commit_desc = reinterpret_cast<CopyDesc*>(base + o_cdesc);
     sp.nlayers = nlayers;
+    sp.nsec = nsec;
     sp.mode = ctx->cfg.mode;
     sp.fuse_commit = ctx->cfg.fuse_commit;
     sp.eps_w = ctx->cfg.eps_w;
@@ -1036,7 +1067,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     ctx->d_commit_desc = sp.commit_desc;
     ctx->d_restore_desc = reinterpret_cast<CopyDesc*>(base + o_rdesc);
 
-    LC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&ctx->h_result), ctx->rl.total, cudaHostAllocDefault));
+    LC_TRY(alloc_host_block(ctx, &ctx->h_result, &ctx->d_h_result));
     ctx->mask.assign(nlayers, 0);
     ctx->offsets.assign(nlayers, 0);
     ctx->state = kReady;
@@ -1211,13 +1242,14 @@ extern "C" lc_status lc_select(lc_ctx* ctx, double tau, int32_t max_staleness, u
     p.tau = tau;
     p.max_staleness = max_staleness;
     p.step = ctx->last_step;
+    p.host_block = ctx->d_h_result;
+    uint32_t* magic = &reinterpret_cast<ResultHeader*>(ctx->h_result)->magic;
+    __atomic_store_n(magic, 0u, __ATOMIC_RELEASE);
     LC_CUDA(launch_select(p, ctx->stream));
     ctx->counters.kernel_launches += 1;
     ctx->counters.select_launches += 1;
-    LC_CUDA(cudaMemcpyAsync(ctx->h_result, ctx->d_result, ctx->rl.total, cudaMemcpyDeviceToHost, ctx->stream));
     ctx->counters.d2h_bytes += ctx->rl.total;
-    LC_CUDA(cudaEventRecord(ctx->ev_result, ctx->stream));
-    LC_TRY(wait_event(ctx->ev_result, ctx->cfg.timeout_ms, "lc_select"));
+    LC_TRY(wait_decision(ctx, magic, "lc_select"));
     LC_TRY(check_copy_fault(ctx, "lc_select"));
 
     ResultHeader h;
@@ -1612,7 +1644,7 @@ extern "C" lc_status lc_wait_durable(lc_ctx* ctx, int64_t step, int32_t timeout_
 namespace {
 
 lc_status ensure_slot_memory(lc_ctx* ctx, lc_ctx::AsyncSlot& sl) {
-    if (!sl.host) LC_CUDA(cudaHostAlloc(reinterpret_cast<void**>(&sl.host), ctx->rl.total, cudaHostAllocDefault));
+    if (!sl.host) LC_TRY(alloc_host_block(ctx, &sl.host, &sl.host_dev));
     if (!sl.done) LC_CUDA(cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming));
     return LC_OK;
 }
@@ -1627,7 +1659,8 @@ lc_status check_step_dst(lc_ctx* ctx, void* dst, uint64_t capacity) {
     return LC_OK;
 }
 
-// Enqueues measure -> select -> pack -> commit -> decision readback on s.
+// Enqueues measure -> select (which writes the decision to host_block, a
+// device address) -> pack -> commit on s.
 lc_status enqueue_step(lc_ctx* ctx, cudaStream_t s, int64_t step, bool step_from_counter, double tau,
                        int32_t max_staleness, uint8_t* dst, uint64_t capacity, uint8_t* host_block) {
     LC_TRY(launch_measure_engine(ctx, s));
@@ -1637,6 +1670,7 @@ lc_status enqueue_step(lc_ctx* ctx, cudaStream_t s, int64_t step, bool step_from
     p.step = step;
     p.step_from_counter = step_from_counter ? 1 : 0;
     p.capacity = capacity;
+    p.host_block = host_block;
     LC_CUDA(launch_select(p, s));
     const ResultHeader* hdr_dev = reinterpret_cast<const ResultHeader*>(ctx->d_result);
     CopyParams c{};
@@ -1659,7 +1693,6 @@ lc_status enqueue_step(lc_ctx* ctx, cudaStream_t s, int64_t step, bool step_from
         k.hi_dev = &hdr_dev->commit_work;
         LC_CUDA(launch_copy_engine(ctx, k, use_bulk(ctx, nullptr), UINT64_MAX, s));
     }
-    LC_CUDA(cudaMemcpyAsync(host_block, ctx->d_result, ctx->rl.total, cudaMemcpyDeviceToHost, s));
     ctx->counters.kernel_launches += 1;
     ctx->counters.select_launches += 1;
     ctx->counters.d2h_bytes += ctx->rl.total;
@@ -1690,7 +1723,7 @@ extern "C" lc_status lc_step_async(lc_ctx* ctx, int64_t step, double tau, int32_
     lc_ctx::AsyncSlot& sl = ctx->slots[free_slot];
     LC_TRY(ensure_slot_memory(ctx, sl));
     LC_TRY(enqueue_step(ctx, ctx->stream, step, false, tau, max_staleness, static_cast<uint8_t*>(dst),
-                        dst_capacity, sl.host));
+                        dst_capacity, sl.host_dev));
     LC_CUDA(cudaEventRecord(sl.done, ctx->stream));
     sl.step = step;
     sl.busy = true;
@@ -1756,7 +1789,7 @@ extern "C" lc_status lc_step_graph_create(lc_ctx* ctx, double tau, int32_t max_s
     const lc_counters before = ctx->counters;
     LC_CUDA(cudaStreamBeginCapture(ctx->capture_stream, cudaStreamCaptureModeThreadLocal));
     lc_status rc = enqueue_step(ctx, ctx->capture_stream, 0, true, tau, max_staleness,
-                                static_cast<uint8_t*>(dst), dst_capacity, sl.host);
+                                static_cast<uint8_t*>(dst), dst_capacity, sl.host_dev);
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(ctx->capture_stream, &graph);
     const lc_counters after = ctx->counters;

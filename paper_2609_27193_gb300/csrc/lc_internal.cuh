@@ -117,8 +117,9 @@ struct SectionDev {
     int32_t idx;          // position among the layer's sections
 };
 
-// Layout of the decision block written by the select kernel and mirrored
-// to pinned host memory.
+// Layout of the decision block that the select kernel writes to pinned host
+// memory: the header (whose magic word comes last), the mask, u and the
+// offsets.  The device keeps a copy of the header for the copies it launches.
 struct ResultHeader {
     int64_t step;
     int32_t n_selected;
@@ -150,6 +151,16 @@ __host__ __device__ inline ResultLayout result_layout(int nlayers) {
     return L;
 }
 
+// A layer's place in the step's packed stream and copy lists.
+struct LayerPlace {
+    uint64_t off;          // of its block in the packed stream
+    uint64_t commit_off;   // of its W sections in the commit work space
+    int32_t pack_idx;      // first pack entry
+    int32_t commit_idx;    // first commit entry
+    int32_t selected;
+    int32_t nwsec;         // its W sections, if selected
+};
+
 struct SelectParams {
     const double* sums;              // [3*nlayers]
     double* delta;                   // [nlayers] accumulators Delta_l
@@ -161,8 +172,9 @@ struct SelectParams {
     const int32_t* layer_wsec_count; // [nlayers] W sections of layer l (first in its range)
     const uint64_t* layer_commit_work; // [nlayers] commit work bytes of layer l's W sections
     const SectionDev* secs;
-    int64_t* layer_scratch;          // [3*nlayers] per-layer output indices
-    uint8_t* result;                 // decision block (device)
+    LayerPlace* layer_place;         // [nlayers]
+    uint8_t* result;                 // header of the decision (device)
+    uint8_t* host_block;             // decision block (device address of pinned host memory)
     CopyDesc* pack_desc;             // [nsec]
     CopyDesc* commit_desc;           // [nseg]
     double* acc_save;                // [nlayers] the step's accumulated drift (for a rollback)
@@ -175,6 +187,7 @@ struct SelectParams {
     int32_t step_from_counter;       // 1: step = *step_counter + 1 (captured graphs)
     int32_t max_staleness;
     int32_t nlayers;
+    int32_t nsec;                    // sections of the layout
     int32_t mode;                    // lc_drift_mode
     int32_t fuse_commit;
 };
