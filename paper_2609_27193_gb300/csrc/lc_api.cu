@@ -366,6 +366,7 @@ struct lc_ctx {
     std::vector<int32_t> layer_seg_begin;  // [nlayers+1]
     std::vector<int64_t> layer_numel;
     std::vector<uint64_t> layer_bytes;
+    uint64_t all_bytes = 0;                // every layer's block
     std::vector<SectionDev> secs;          // packed order, layer-major
     std::vector<int32_t> layer_sec_begin;  // [nlayers+1]
     std::vector<int32_t> sec_seg;          // segment (measure order) of each section
@@ -499,12 +500,14 @@ bool use_bulk(const lc_ctx* ctx, const void* base) {
     return ctx->cfg.copy_engine == LC_COPY_BULK && ctx->bulk_sources && (!base || plain_device(base));
 }
 
-cudaError_t launch_copy_engine(lc_ctx* ctx, CopyParams p, bool bulk, uint64_t units, cudaStream_t s) {
+// `bytes`: the launch's range, or a bound on it where the device decides.
+cudaError_t launch_copy_engine(lc_ctx* ctx, CopyParams p, bool bulk, uint64_t bytes, cudaStream_t s) {
     p.fault = ctx->d_fault;
     p.fault_dev = ctx->d_fault_dev;
     p.stall_first = (ctx->cfg.debug_flags & LC_DEBUG_BULK_STALL) ? 1 : 0;
     const uint64_t cap = uint64_t(bulk ? ctx->bulk_grid : ctx->copy_grid);
-    const int grid = int(std::max<uint64_t>(1, std::min<uint64_t>(cap, units)));
+    p.resident = bulk ? ctx->bulk_grid / LC_COPY_BULK_WAVES : ctx->copy_grid;
+    const int grid = int(std::max<uint64_t>(1, std::min(copy_shares(bytes, uint64_t(p.resident), cap), bytes >> 4)));
     ctx->counters.kernel_launches += 1;
     ctx->counters.copy_launches += 1;
     if (bulk) ctx->counters.bulk_copy_launches += 1;
@@ -931,6 +934,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
             }
         }
         ctx->layer_bytes[l] = off;
+        ctx->all_bytes += off;
     }
     ctx->layer_sec_begin[nlayers] = int32_t(ctx->secs.size());
     const int32_t nsec = int32_t(ctx->secs.size());
@@ -1310,7 +1314,7 @@ lc_status launch_copy_range(lc_ctx* ctx, const CopyDesc* desc, int ndesc, int mo
     p.base = base;
     p.ndesc_dev = nullptr;
     p.hi_dev = nullptr;
-    LC_CUDA(launch_copy_engine(ctx, p, use_bulk(ctx, base), (hi - lo) >> 4, s));
+    LC_CUDA(launch_copy_engine(ctx, p, use_bulk(ctx, base), hi - lo, s));
     return LC_OK;
 }
 
@@ -1682,8 +1686,10 @@ lc_status enqueue_step(lc_ctx* ctx, cudaStream_t s, int64_t step, bool step_from
     c.base = dst;
     c.ndesc_dev = &hdr_dev->n_pack_desc;
     c.hi_dev = &hdr_dev->pack_bytes;
-    // sizes are decided on the device: full grids, idle CTAs return at once
-    LC_CUDA(launch_copy_engine(ctx, c, use_bulk(ctx, dst), UINT64_MAX, s));
+    // sizes are decided on the device: grids for the most that can be selected,
+    // idle CTAs return at once
+    const uint64_t most = std::min(capacity, ctx->all_bytes);
+    LC_CUDA(launch_copy_engine(ctx, c, use_bulk(ctx, dst), most, s));
     if (ctx->cfg.mode == LC_DRIFT_SNAPSHOT && !ctx->cfg.fuse_commit) {
         CopyParams k = c;
         k.desc = ctx->d_commit_desc;
@@ -1691,7 +1697,7 @@ lc_status enqueue_step(lc_ctx* ctx, cudaStream_t s, int64_t step, bool step_from
         k.base = nullptr;
         k.ndesc_dev = &hdr_dev->n_commit_desc;
         k.hi_dev = &hdr_dev->commit_work;
-        LC_CUDA(launch_copy_engine(ctx, k, use_bulk(ctx, nullptr), UINT64_MAX, s));
+        LC_CUDA(launch_copy_engine(ctx, k, use_bulk(ctx, nullptr), most, s));
     }
     ctx->counters.kernel_launches += 1;
     ctx->counters.select_launches += 1;

@@ -8,8 +8,8 @@
 //
 // A launch covers the work range [lo, hi) of a descriptor list whose
 // entries tile a linear work space (lc_internal.cuh).  The range is cut into
-// G equal 16-byte-aligned pieces, one per CTA; a CTA finds its first entry
-// by binary search and walks the entries it overlaps.  Within an entry the
+// equal 16-byte-aligned pieces, one per CTA; a CTA finds its first entry by a
+// search over the warp and walks the entries it overlaps.  Within an entry the
 // payload moves in 16-byte vectors when source and destinations are all
 // 16-byte aligned (the usual case: torch allocations, 256-byte packed
 // sections), else in the widest unit the three addresses share.  In GATHER
@@ -164,9 +164,24 @@ __device__ void copy_entry(const CopyParams& p, const CopyDesc& d, uint64_t a, u
     }
 }
 
+// The last of n entries with woff <= x (the first one has), searched by a
+// warp: 32 places a step instead of two, since every step waits for a load.
+__device__ __forceinline__ int find_entry(const CopyDesc* desc, int n, uint64_t x) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 1) {
+        const int step = (n + 31) / 32, i = lane * step;
+        const unsigned int below = __ballot_sync(0xffffffffu, i < n && desc[lo + (i < n ? i : 0)].woff <= x);
+        const int k = (__popc(below) - 1) * step;
+        lo += k;
+        n = n - k < step ? n - k : step;
+    }
+    return lo;
+}
+
 // The CTA's work range [x, xe) (granules of LC_COPY_ALIGN_BYTES, the last
 // one ragged) and the last entry with woff <= x.  Returns false when the
-// CTA has nothing to do.
+// CTA has nothing to do.  Called by whole warps.
 __device__ __forceinline__ bool cta_range(CopyParams& p, uint64_t& x, uint64_t& xe, int& first) {
     if (p.ndesc_dev) {           // sizes decided on the device by the select kernel
         p.ndesc = *p.ndesc_dev;
@@ -175,19 +190,15 @@ __device__ __forceinline__ bool cta_range(CopyParams& p, uint64_t& x, uint64_t& 
     constexpr uint64_t kGran = LC_COPY_ALIGN_BYTES / 16;
     const uint64_t units = (p.hi - p.lo) >> 4;
     const uint64_t grans = (units + kGran - 1) / kGran;
-    const uint64_t u0 = grans * blockIdx.x / gridDim.x * kGran;
-    uint64_t u1 = grans * (blockIdx.x + 1) / gridDim.x * kGran;
+    const uint64_t shares = copy_shares(p.hi - p.lo, uint64_t(p.resident), gridDim.x);
+    if (blockIdx.x >= shares) return false;
+    const uint64_t u0 = grans * blockIdx.x / shares * kGran;
+    uint64_t u1 = grans * (blockIdx.x + 1) / shares * kGran;
     if (u1 > units) u1 = units;
     if (u0 >= u1 || p.ndesc <= 0) return false;
     x = p.lo + (u0 << 4);
     xe = p.lo + (u1 << 4);
-    int lo_i = 0, hi_i = p.ndesc - 1;
-    while (lo_i < hi_i) {
-        const int mid = (lo_i + hi_i + 1) >> 1;
-        if (p.desc[mid].woff <= x) lo_i = mid;
-        else hi_i = mid - 1;
-    }
-    first = lo_i;
+    first = find_entry(p.desc, p.ndesc, x);
     return true;
 }
 
