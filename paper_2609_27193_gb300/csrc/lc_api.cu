@@ -8,6 +8,7 @@
 #include "layercheck.h"
 #include "lc_host.h"
 #include "lc_internal.cuh"
+#include "lc_partition.cuh"
 
 #include <nvtx3/nvToolsExt.h>
 
@@ -28,28 +29,11 @@
 
 using namespace lc;
 
-// CTAs of a bulk-engine launch, in waves of one CTA per resident slot.  With
+// CTAs of a bulk-engine copy, in waves of one CTA per resident slot.  With
 // more than one wave each CTA takes a smaller share of the range, and SMs
 // that finish early start the next CTAs, which shortens the launch's tail.
-#ifndef LC_MEASURE_BULK_WAVES
-#define LC_MEASURE_BULK_WAVES 1
-#endif
 #ifndef LC_COPY_BULK_WAVES
 #define LC_COPY_BULK_WAVES 8
-#endif
-// The bulk measure (and the fused step on its partition): a CTA walks an
-// equal share of the first (100 - LC_MEASURE_POOL_PCT)% of the work space,
-// then takes small units of the rest, LC_MEASURE_POOL_UNITS per CTA in all,
-// from a counter.  CTAs that stream faster take more units, so the launch
-// ends when the pool runs dry rather than when its slowest share is done.
-#ifndef LC_MEASURE_POOL_PCT
-#define LC_MEASURE_POOL_PCT 10
-#endif
-#ifndef LC_MEASURE_POOL_MIN
-#define LC_MEASURE_POOL_MIN 1024
-#endif
-#ifndef LC_MEASURE_POOL_UNITS
-#define LC_MEASURE_POOL_UNITS 8
 #endif
 
 // ---------------------------------------------------------------------------
@@ -828,67 +812,31 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         d.vec_begin = V;
         V += d.nvec;
     }
-    // CTA work ranges of the measure work space: G equal shares in granules
-    // of LC_MEASURE_ALIGN_VECS, and a partial slot for every (range, layer) run
-    // (with a pool: G static ranges over the first granules, then `units`
-    // ranges over the rest; range r's slots are fixed whichever CTA walks it)
     struct Partition {
-        int64_t G = 0;
-        int64_t units = 0;
+        PartitionShape sh;
         std::vector<int64_t> cta_vec;
         std::vector<int32_t> cta_seg0, cta_slot0, layer_slot_begin;
         int32_t nslots = 0;
     };
-    auto partition = [&](int64_t grid, int64_t pool_pct = 0, int64_t units_per_cta = 0) {
+    auto partition = [&](int64_t grid, bool with_pool) {
         Partition pt;
-        const int64_t gran = LC_MEASURE_ALIGN_VECS;
-        const int64_t ngran = (V + gran - 1) / gran;
-        pt.G = std::max<int64_t>(1, std::min<int64_t>(ngran, grid));
-        const int64_t G = pt.G;
-        // granules in the pool, in units of at least kMinUnit granules (512 KB
-        // of W: a unit costs a counter fetch, a table lookup and a flush); a
-        // pool too small to give every CTA a unit on average is not used
-        constexpr int64_t kMinUnit = LC_MEASURE_POOL_MIN;
-        int64_t pool = pool_pct > 0 ? ngran * pool_pct / 100 : 0;
-        pt.units = pool >= G * kMinUnit ? std::min<int64_t>(G * units_per_cta, pool / kMinUnit) : 0;
-        if (pt.units == 0) pool = 0;
-        const int64_t U = pt.units, R = G + U, ng_static = ngran - pool;
+        pt.sh = partition_shape(V, grid, with_pool);
+        const size_t R = size_t(pt.sh.ranges());
         pt.cta_vec.resize(R + 1);
         pt.cta_seg0.resize(R);
         pt.cta_slot0.resize(R);
-        pt.layer_slot_begin.assign(nlayers + 1, -1);
-        for (int64_t b = 0; b <= G; ++b) pt.cta_vec[b] = std::min(V, ng_static * b / G * gran);
-        for (int64_t u = 1; u <= U; ++u) pt.cta_vec[G + u] = std::min(V, (ng_static + pool * u / U) * gran);
-        int32_t slot = 0, s = 0;
-        for (int64_t b = 0; b < R; ++b) {
-            const int64_t v0 = pt.cta_vec[b], v1 = pt.cta_vec[b + 1];
-            while (s < nseg && sd[s].vec_begin + sd[s].nvec <= v0) ++s;
-            pt.cta_seg0[b] = s;
-            pt.cta_slot0[b] = slot;
-            // one slot per layer of the range; ranges and layers both follow
-            // the work space, so a layer's slots are contiguous
-            for (int32_t t = s; v0 < v1 && t < nseg && sd[t].vec_begin < v1; ++t) {
-                if (t > s && sd[t].layer == sd[t - 1].layer) continue;
-                int32_t& first = pt.layer_slot_begin[sd[t].layer];
-                if (first < 0) first = slot;
-                ++slot;
-            }
-        }
-        pt.layer_slot_begin[nlayers] = slot;
-        for (int32_t l = nlayers - 1; l >= 0; --l)
-            if (pt.layer_slot_begin[l] < 0) pt.layer_slot_begin[l] = pt.layer_slot_begin[l + 1];
-        pt.nslots = slot;
+        pt.layer_slot_begin.resize(size_t(nlayers) + 1);
+        pt.nslots = partition_fill(pt.sh, sd.data(), nseg, nlayers, pt.cta_vec.data(), pt.cta_seg0.data(),
+                                   pt.cta_slot0.data(), pt.layer_slot_begin.data());
         return pt;
     };
     int occ = 0;
     LC_CUDA(measure_occupancy(&occ));
-    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ));
+    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ), false);
     int bocc = 0;
     LC_CUDA(measure_bulk_prepare(&bocc));
-    const Partition pb = partition(int64_t(ctx->sms) * std::max(1, bocc) * LC_MEASURE_BULK_WAVES,
-                                   LC_MEASURE_POOL_PCT, LC_MEASURE_POOL_UNITS);
-    const int64_t Rb = pb.G + pb.units;
-    const int64_t G = pa.G, Gb = pb.G;
+    const Partition pb = partition(int64_t(ctx->sms) * std::max(1, bocc) * LC_MEASURE_BULK_WAVES, true);
+    const int64_t Rb = pb.sh.ranges(), G = pa.sh.G, Gb = pb.sh.G;
     ctx->measure_grid = int(G);
     ctx->measure_bulk_grid = int(Gb);
     ctx->nslots = pa.nslots;
@@ -1035,8 +983,8 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     mpb.layer_slot_begin = reinterpret_cast<const int32_t*>(base + o_lslot_b);
     mpb.partials = reinterpret_cast<double2*>(base + o_part_b);
     mpb.ticket = reinterpret_cast<unsigned int*>(base + o_ticket_b);
-    mpb.units = int32_t(pb.units);
-    ctx->counters.measure_pool_units = pb.units;
+    mpb.units = int32_t(pb.sh.units);
+    ctx->counters.measure_pool_units = pb.sh.units;
     mpb.unit_next = reinterpret_cast<unsigned int*>(base + o_unit_b);
     mpb.stall_first = (ctx->cfg.debug_flags & LC_DEBUG_MEASURE_STALL) ? 1 : 0;
     ctx->bulk_measure = ctx->cfg.copy_engine == LC_COPY_BULK && all_device && !ctx->snap_missing;

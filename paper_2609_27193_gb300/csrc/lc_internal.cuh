@@ -61,6 +61,9 @@ struct MeasureParams {
     // atomicAdd(unit_next, 1), until the pool is empty; 0: no pool
     int32_t units;
     unsigned int* unit_next;         // reset by the last CTA
+    // 1: a fault turns every sum into NaN (for a caller that has no status to
+    // read it from); `fault` is device memory then
+    int32_t nan_on_fault;
 };
 
 // One copy entry.  The entries of a launch tile a linear "work space"

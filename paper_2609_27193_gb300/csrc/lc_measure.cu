@@ -628,6 +628,10 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
     __threadfence();
     // the ring's loads have all landed (or the CTA gave up): it stages the combine
     finalize(p, reinterpret_cast<double2*>(ring), int32_t(kMeasureBulkSmem / sizeof(double2)), &tables);
+    if (p.nan_on_fault && *reinterpret_cast<volatile const uint32_t*>(p.fault)) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < 3 * p.nlayers; i += blockDim.x) p.sums[i] = __longlong_as_double(-1);
+    }
 }
 
 }  // namespace

@@ -1,20 +1,22 @@
 // lc_noalloc.cu -- lc_measure_noalloc: the per-layer sums of lc_measure for
 // callers that cannot allocate device memory.
 //
-// It launches the same measure kernel as lc_measure, but every table and
-// scratch buffer that kernel needs (segment table, CTA partition, partial
-// sums, completion counter) lives in one file-scope static device array of
+// It launches the same measure kernels as lc_measure (the bulk-load one when
+// every W and R is cudaMalloc memory), on the same partition, but every table
+// and scratch buffer that they need (segment table, partition, partial sums,
+// counters) lives in one file-scope static device array of
 // LC_NOALLOC_SCRATCH_BYTES.  Host code never uses the array's name as an
 // address: at set-up, once per device and with that device current, the
 // array's device address is looked up with cudaGetSymbolAddress and cached.
 // The tables are built on the host and reach the array as the kernel
 // parameters of small upload kernels launched on the caller's stream ahead
 // of the measure, so the driver copies them when each upload is launched and
-// nothing reads host memory once the call has returned.  The completion
-// counter travels in the upload as zero.  No cudaMalloc, cudaFree or other
+// nothing reads host memory once the call has returned.  The counters and the
+// fault word travel in the upload as zeros.  No cudaMalloc, cudaFree or other
 // allocating routine is called.
 #include "layercheck.h"
 #include "lc_internal.cuh"
+#include "lc_partition.cuh"
 
 #include <cstdarg>
 #include <cstdio>
@@ -27,7 +29,7 @@ namespace {
 
 constexpr int kMaxSeg = LC_NOALLOC_MAX_SEGMENTS;
 constexpr int kMaxLayers = LC_NOALLOC_MAX_LAYERS;
-constexpr int kMaxCtas = 2048;
+constexpr int kMaxRanges = 4096;
 constexpr int kMaxDevices = 64;
 
 constexpr size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -38,26 +40,26 @@ constexpr size_t al16(size_t x) { return (x + 15) & ~size_t(15); }
 // back to back (16-byte aligned) for the call's sizes, so the upload moves
 // only the bytes the measure will read.
 struct TableLayout {
-    size_t segs, cta_vec, layer_n, cta_seg, cta_slot, layer_slot, ticket, bytes;
+    size_t segs, cta_vec, layer_n, cta_seg, cta_slot, layer_slot, counters, bytes;
 };
 
-constexpr TableLayout table_layout(size_t nseg, size_t nlayers, size_t G) {
+constexpr TableLayout table_layout(size_t nseg, size_t nlayers, size_t R) {
     TableLayout t{};
     t.segs = 0;
     t.cta_vec = al16(t.segs + sizeof(SegDev) * nseg);
-    t.layer_n = al16(t.cta_vec + sizeof(int64_t) * (G + 1));
+    t.layer_n = al16(t.cta_vec + sizeof(int64_t) * (R + 1));
     t.cta_seg = al16(t.layer_n + sizeof(double) * nlayers);
-    t.cta_slot = al16(t.cta_seg + sizeof(int32_t) * G);
-    t.layer_slot = al16(t.cta_slot + sizeof(int32_t) * G);
-    t.ticket = al16(t.layer_slot + sizeof(int32_t) * (nlayers + 1));
-    t.bytes = al16(t.ticket + sizeof(unsigned int));
+    t.cta_slot = al16(t.cta_seg + sizeof(int32_t) * R);
+    t.layer_slot = al16(t.cta_slot + sizeof(int32_t) * R);
+    t.counters = al16(t.layer_slot + sizeof(int32_t) * (nlayers + 1));   // completion, pool, fault word
+    t.bytes = al16(t.counters + 3 * sizeof(unsigned int));
     return t;
 }
 
 // Scratch layout: the tables (at most kTableBytes), then the kernel scratch.
-constexpr size_t kTableBytes = al256(table_layout(kMaxSeg, kMaxLayers, kMaxCtas).bytes);
+constexpr size_t kTableBytes = al256(table_layout(kMaxSeg, kMaxLayers, kMaxRanges).bytes);
 constexpr size_t kOffPartials = kTableBytes;
-constexpr size_t kScratchUsed = al256(kOffPartials + sizeof(double2) * (kMaxCtas + kMaxLayers));
+constexpr size_t kScratchUsed = al256(kOffPartials + sizeof(double2) * (kMaxRanges + kMaxLayers));
 static_assert(kScratchUsed <= LC_NOALLOC_SCRATCH_BYTES, "scratch layout exceeds its array");
 
 }  // namespace
@@ -70,13 +72,15 @@ namespace {
 // One upload: `nbytes` (a multiple of 16) of the table image, to be written
 // at byte `dst_off` of the scratch array.  Passed by value, so the launch
 // itself carries the bytes.
-constexpr int kUploadVecs = 1024;   // 16 KB of payload per launch
+// 31.75 KB of payload per launch, what kernel parameters hold: one launch for
+// the tables of up to about 300 segments.
+constexpr int kUploadVecs = 2032;
 struct UploadChunk {
     uint32_t dst_off;
     uint32_t nbytes;
     uint4 data[kUploadVecs];
 };
-static_assert(sizeof(UploadChunk) <= 32000, "kernel parameters are limited to 32764 bytes");
+static_assert(sizeof(UploadChunk) <= 32764, "kernel parameters are limited to 32764 bytes");
 
 __global__ void __launch_bounds__(256) noalloc_upload_kernel(const __grid_constant__ UploadChunk c) {
     uint4* dst = reinterpret_cast<uint4*>(g_noalloc_scratch + c.dst_off);
@@ -91,7 +95,8 @@ namespace {
 struct DeviceScratch {
     bool ready = false;
     unsigned char* addr = nullptr;   // device address of g_noalloc_scratch
-    int max_grid = 0;
+    int max_grid = 0;                // resident CTAs of the thread kernel
+    int bulk_grid = 0;               // and of the bulk-load kernel
 };
 DeviceScratch g_scratch[kMaxDevices];
 std::mutex g_scratch_mu;
@@ -138,30 +143,37 @@ lc_status setup_device(int device, DeviceScratch* out) {
             return err(LC_ERR_CUDA, "lc_measure_noalloc: cudaGetSymbolAddress failed: %s",
                        cudaGetErrorString(e));
         }
-        int sms = 0, occ = 0;
+        int sms = 0, occ = 0, bocc = 0;
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
         if (e == cudaSuccess) e = measure_occupancy(&occ);
+        if (e == cudaSuccess) e = measure_bulk_prepare(&bocc);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return err(LC_ERR_CUDA, "lc_measure_noalloc: device query failed: %s", cudaGetErrorString(e));
         }
         d.addr = static_cast<unsigned char*>(addr);
         d.max_grid = sms * (occ > 0 ? occ : 1);
-        if (d.max_grid > kMaxCtas) d.max_grid = kMaxCtas;
-        if (d.max_grid < 1) d.max_grid = 1;
+        if (d.max_grid > kMaxRanges) d.max_grid = kMaxRanges;
+        // room for the pool's ranges too
+        d.bulk_grid = sms * (bocc > 0 ? bocc : 1) * LC_MEASURE_BULK_WAVES;
+        if (d.bulk_grid > kMaxRanges / (1 + LC_MEASURE_POOL_UNITS)) d.bulk_grid = kMaxRanges / (1 + LC_MEASURE_POOL_UNITS);
         d.ready = true;
     }
     *out = d;
     return LC_OK;
 }
 
-bool is_device_memory(const void* p, int device) {
+// `plain` becomes false for managed memory, which the bulk engine is not given.
+bool is_device_memory(const void* p, int device, bool* plain) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    if (a.type == cudaMemoryTypeManaged) return true;
+    if (a.type == cudaMemoryTypeManaged) {
+        *plain = false;
+        return true;
+    }
     return a.type == cudaMemoryTypeDevice && a.device == device;
 }
 
@@ -189,7 +201,9 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: device %d out of range", device);
     CurrentDevice cur(device);
     if (!cur.ok) return err(LC_ERR_CUDA, "lc_measure_noalloc: cannot make device %d current", device);
-    if (!is_device_memory(sums_out, device))
+    bool bulk = true;
+    bool sums_plain = true;
+    if (!is_device_memory(sums_out, device, &sums_plain))
         return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: sums_out is not device memory");
 
     // validate and order the segments: layers ascending, registration order within
@@ -209,7 +223,7 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         const uintptr_t esz = s.w_dtype == LC_BF16 ? 2 : 4;
         if ((reinterpret_cast<uintptr_t>(s.w) % esz) || (reinterpret_cast<uintptr_t>(s.snap) % esz))
             return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: segment %d not element-aligned", i);
-        if (!is_device_memory(s.w, device) || !is_device_memory(s.snap, device))
+        if (!is_device_memory(s.w, device, &bulk) || !is_device_memory(s.snap, device, &bulk))
             return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: segment %d is not device memory", i);
         per_layer[s.layer] += 1;
     }
@@ -223,7 +237,6 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
     lc_status st = setup_device(device, &ds);
     if (st != LC_OK) return st;
 
-    std::memset(t_image, 0, sizeof t_image);
     // the segment table sits at offset 0 whatever the grid; the rest of the
     // layout depends on the grid, known once the work space is measured
     SegDev* sd = reinterpret_cast<SegDev*>(t_image);
@@ -248,41 +261,20 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         sd[i].vec_begin = V;
         V += sd[i].nvec;
     }
-    const int64_t ngran = (V + LC_MEASURE_ALIGN_VECS - 1) / LC_MEASURE_ALIGN_VECS;
-    const int64_t G = ngran < ds.max_grid ? ngran : ds.max_grid;
-    const TableLayout L = table_layout(size_t(nseg), size_t(nlayers), size_t(G));
-    if (L.bytes > kTableBytes) return err(LC_ERR_CUDA, "lc_measure_noalloc: internal table overflow");
-    int64_t* cta_vec = reinterpret_cast<int64_t*>(t_image + L.cta_vec);
-    int32_t* cta_seg = reinterpret_cast<int32_t*>(t_image + L.cta_seg);
-    int32_t* cta_slot = reinterpret_cast<int32_t*>(t_image + L.cta_slot);
-    int32_t* layer_slot = reinterpret_cast<int32_t*>(t_image + L.layer_slot);
+    const PartitionShape sh = partition_shape(V, bulk ? ds.bulk_grid : ds.max_grid, bulk);
+    const TableLayout L = table_layout(size_t(nseg), size_t(nlayers), size_t(sh.ranges()));
+    if (sh.ranges() > kMaxRanges || L.bytes > kTableBytes)
+        return err(LC_ERR_CUDA, "lc_measure_noalloc: internal table overflow");
     double* layer_n = reinterpret_cast<double*>(t_image + L.layer_n);
-    for (int32_t l = 0; l <= nlayers; ++l) layer_slot[l] = -1;
     for (int32_t l = 0; l < nlayers; ++l) {
         int64_t n = 0;
         for (int32_t i = layer_begin[l]; i < layer_begin[l + 1]; ++i) n += sd[i].numel;
         layer_n[l] = double(n);
     }
-    for (int64_t b = 0; b <= G; ++b) {
-        const int64_t v = ngran * b / G * LC_MEASURE_ALIGN_VECS;
-        cta_vec[b] = v < V ? v : V;
-    }
-    int32_t slot = 0, s = 0;
-    for (int64_t b = 0; b < G; ++b) {
-        const int64_t v0 = cta_vec[b], v1 = cta_vec[b + 1];
-        while (s < nseg && sd[s].vec_begin + sd[s].nvec <= v0) ++s;
-        cta_seg[b] = s;
-        cta_slot[b] = slot;
-        for (int32_t t = s; v0 < v1 && t < nseg && sd[t].vec_begin < v1; ++t) {
-            if (t > s && sd[t].layer == sd[t - 1].layer) continue;
-            if (layer_slot[sd[t].layer] < 0) layer_slot[sd[t].layer] = slot;
-            ++slot;
-        }
-    }
-    layer_slot[nlayers] = slot;
-    for (int32_t l = nlayers - 1; l >= 0; --l)
-        if (layer_slot[l] < 0) layer_slot[l] = layer_slot[l + 1];
-    if (slot > kMaxCtas + kMaxLayers) return err(LC_ERR_CUDA, "lc_measure_noalloc: internal slot overflow");
+    partition_fill(sh, sd, nseg, nlayers, reinterpret_cast<int64_t*>(t_image + L.cta_vec),
+                   reinterpret_cast<int32_t*>(t_image + L.cta_seg), reinterpret_cast<int32_t*>(t_image + L.cta_slot),
+                   reinterpret_cast<int32_t*>(t_image + L.layer_slot));
+    std::memset(t_image + L.counters, 0, 3 * sizeof(unsigned int));
 
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
     // the tables and a zero completion counter into the scratch array,
@@ -307,10 +299,16 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
     p.layer_n = reinterpret_cast<const double*>(ds.addr + L.layer_n);
     p.partials = reinterpret_cast<double2*>(ds.addr + kOffPartials);
     p.sums = sums_out;
-    p.ticket = reinterpret_cast<unsigned int*>(ds.addr + L.ticket);
+    unsigned int* counters = reinterpret_cast<unsigned int*>(ds.addr + L.counters);
+    p.ticket = counters;
+    p.unit_next = counters + 1;
+    p.units = int32_t(sh.units);
+    p.fault = counters + 2;
+    p.nan_on_fault = 1;
     p.nseg = nseg;
     p.nlayers = nlayers;
-    const cudaError_t e = launch_measure(p, int(G), false, stream);
+    const cudaError_t e = bulk ? launch_measure_bulk(p, int(sh.G), false, stream)
+                               : launch_measure(p, int(sh.G), false, stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return err(LC_ERR_CUDA, "lc_measure_noalloc: launch failed: %s", cudaGetErrorString(e));

@@ -1,0 +1,91 @@
+// lc_partition.cuh -- host side of the measure's work partition, shared by
+// the contexts (lc_api.cu) and the allocation-free measure (lc_noalloc.cu).
+#pragma once
+
+#include "lc_internal.cuh"
+
+#include <stddef.h>
+#include <stdint.h>
+
+// CTAs of a bulk-engine measure, in waves of one CTA per resident slot.
+#ifndef LC_MEASURE_BULK_WAVES
+#define LC_MEASURE_BULK_WAVES 1
+#endif
+// The bulk measure (and the fused step on its partition): a CTA walks an
+// equal share of the first (100 - LC_MEASURE_POOL_PCT)% of the work space,
+// then takes small units of the rest, LC_MEASURE_POOL_UNITS per CTA in all,
+// from a counter.  CTAs that stream faster take more units, so the launch
+// ends when the pool runs dry rather than when its slowest share is done.
+// A unit is at least LC_MEASURE_POOL_MIN granules (512 KB of W: it costs a
+// counter fetch, a table lookup and a flush); a pool too small to give every
+// CTA a unit on average is not used.
+#ifndef LC_MEASURE_POOL_PCT
+#define LC_MEASURE_POOL_PCT 10
+#endif
+#ifndef LC_MEASURE_POOL_MIN
+#define LC_MEASURE_POOL_MIN 1024
+#endif
+#ifndef LC_MEASURE_POOL_UNITS
+#define LC_MEASURE_POOL_UNITS 8
+#endif
+
+namespace lc {
+
+// G equal shares of the work space in granules of LC_MEASURE_ALIGN_VECS and,
+// with a pool, `units` ranges over what the shares leave.
+struct PartitionShape {
+    int64_t V = 0;        // vectors of the work space
+    int64_t ngran = 0;    // granules
+    int64_t pool = 0;     // granules in the pool
+    int64_t G = 1;        // ranges that are a CTA's own
+    int64_t units = 0;    // ranges in the pool
+    int64_t ranges() const { return G + units; }
+};
+
+inline PartitionShape partition_shape(int64_t V, int64_t grid, bool with_pool) {
+    PartitionShape s;
+    s.V = V;
+    s.ngran = (V + LC_MEASURE_ALIGN_VECS - 1) / LC_MEASURE_ALIGN_VECS;
+    s.G = s.ngran < grid ? s.ngran : grid;
+    if (s.G < 1) s.G = 1;
+    if (with_pool) {
+        const int64_t pool = s.ngran * LC_MEASURE_POOL_PCT / 100, most = s.G * LC_MEASURE_POOL_UNITS;
+        if (pool >= s.G * LC_MEASURE_POOL_MIN) {
+            s.units = pool / LC_MEASURE_POOL_MIN < most ? pool / LC_MEASURE_POOL_MIN : most;
+            s.pool = pool;
+        }
+    }
+    return s;
+}
+
+// Fills the ranges' tables (vec: ranges() + 1; seg0, slot0: ranges()) and the
+// layers' slots (layer_slot: nlayers + 1) for segments in measure order;
+// returns the number of slots, at most ranges() + nlayers.  One slot per
+// (range, layer) run: ranges and layers both follow the work space, so a
+// layer's slots are contiguous, and a range's are fixed whichever CTA walks it.
+inline int32_t partition_fill(const PartitionShape& sh, const SegDev* sd, int32_t nseg, int32_t nlayers, int64_t* vec,
+                              int32_t* seg0, int32_t* slot0, int32_t* layer_slot) {
+    const int64_t gran = LC_MEASURE_ALIGN_VECS, own = sh.ngran - sh.pool, R = sh.ranges();
+    auto at = [&](int64_t g) { return g * gran < sh.V ? g * gran : sh.V; };
+    for (int64_t b = 0; b <= sh.G; ++b) vec[b] = at(own * b / sh.G);
+    for (int64_t u = 1; u <= sh.units; ++u) vec[sh.G + u] = at(own + sh.pool * u / sh.units);
+    for (int32_t l = 0; l < nlayers; ++l) layer_slot[l] = -1;
+    int32_t slot = 0, s = 0;
+    for (int64_t b = 0; b < R; ++b) {
+        const int64_t v0 = vec[b], v1 = vec[b + 1];
+        while (s < nseg && sd[s].vec_begin + sd[s].nvec <= v0) ++s;
+        seg0[b] = s;
+        slot0[b] = slot;
+        for (int32_t t = s; v0 < v1 && t < nseg && sd[t].vec_begin < v1; ++t) {
+            if (t > s && sd[t].layer == sd[t - 1].layer) continue;
+            if (layer_slot[sd[t].layer] < 0) layer_slot[sd[t].layer] = slot;
+            ++slot;
+        }
+    }
+    layer_slot[nlayers] = slot;
+    for (int32_t l = nlayers - 1; l >= 0; --l)
+        if (layer_slot[l] < 0) layer_slot[l] = layer_slot[l + 1];
+    return slot;
+}
+
+}  // namespace lc

@@ -234,3 +234,37 @@ def test_adamw_off_alignment(lead, grad_dtype):
     assert (np.abs(got - want) <= 5 * 2.0 ** -24 * np.abs(want)).all()
     assert lc.counters()["bulk_measure_launches"] == 1
     lc.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_noalloc_measure_off_alignment(dtype):
+    """lc_measure_noalloc over references at every offset from the weights,
+    sizes at the ends of vectors and chunks, layers in shuffled order: exact
+    sums, and again on the next call with other values."""
+    torch = require_gpu()
+    import ctypes as C
+    import paper_2609_27193_gb300 as P
+    from paper_2609_27193_gb300 import _abi
+    esz = 2 if dtype == "bf16" else 4
+    tt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    g = torch.Generator(device="cuda").manual_seed(esz)
+    keep = []
+    for n in SIZES:
+        for shift in range(0, 16, esz):
+            lead = esz * (len(keep) % (16 // esz))
+            keep.append((_placed(torch, n, tt, lead)[1], _placed(torch, n, tt, (lead + shift) % 16)[1]))
+    N = len(keep)
+    order = np.random.default_rng(esz).permutation(N)
+    segs = (_abi.lc_segment * N)(*[P.segment(int(k), *keep[k]) for k in order])
+    out = torch.empty(3 * N, dtype=torch.float64, device="cuda")
+    for _ in range(2):
+        for w, r in keep:
+            w.copy_(_grid(torch, w.numel(), g))
+            r.copy_(_grid(torch, w.numel(), g))
+        out.fill_(float("nan"))
+        _abi.check(P.library().lc_measure_noalloc(0, C.c_void_p(torch.cuda.current_stream().cuda_stream), segs, N, N,
+                                                  C.c_void_p(out.data_ptr())))
+        got = out.cpu().numpy().reshape(N, 3)
+        for k, (w, r) in enumerate(keep):
+            d, a = (w.double() - r.double()).abs().sum().item(), r.double().abs().sum().item()
+            assert got[k].tolist() == [d, a, w.numel()], (k, w.numel())
