@@ -16,14 +16,17 @@
 // then takes small units of the rest, LC_MEASURE_POOL_UNITS per CTA in all,
 // from a counter.  CTAs that stream faster take more units, so the launch
 // ends when the pool runs dry rather than when its slowest share is done.
-// A unit is at least LC_MEASURE_POOL_MIN granules (512 KB of W: it costs a
+// A unit is at least LC_MEASURE_POOL_MIN granules (64 KB of W: it costs a
 // counter fetch, a table lookup and a flush); a pool too small to give every
-// CTA a unit on average is not used.
+// CTA a unit on average is not used.  With units of 512 KB (before a flush
+// cost five fp64 adds a warp instead of ten) the fused step over 1.2 G
+// parameters takes 5196 instead of 5162 us, the measure of 412 M 256 instead of
+// 253, of 138 M fp32 parameters 179 instead of 177; 64 to 256 KB are alike.
 #ifndef LC_MEASURE_POOL_PCT
 #define LC_MEASURE_POOL_PCT 10
 #endif
 #ifndef LC_MEASURE_POOL_MIN
-#define LC_MEASURE_POOL_MIN 1024
+#define LC_MEASURE_POOL_MIN 128
 #endif
 #ifndef LC_MEASURE_POOL_UNITS
 #define LC_MEASURE_POOL_UNITS 8
