@@ -635,6 +635,8 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) adamw_bulk_kernel(const Me
         mbar_init_fence();
     }
     fin_prefetch(p, tables);
+    dependents_may_start();
+    dependency_wait();
     __syncthreads();
     if (threadIdx.x == 0) {
         adam_produce(p, opt, ring, r);
@@ -667,9 +669,7 @@ cudaError_t launch_adamw_measure(const MeasureParams& p, const OptSegDev* opt, c
 
 cudaError_t launch_adamw_bulk(const MeasureParams& p, const OptSegDev* opt, const AdamConsts& c, int grid,
                               cudaStream_t s) {
-    cudaGetLastError();
-    adamw_bulk_kernel<<<grid, kMeasureThreads, kAdamBulkSmem, s>>>(p, opt, c);
-    return cudaGetLastError();
+    return launch_dependent(adamw_bulk_kernel, grid, kMeasureThreads, kAdamBulkSmem, s, p, opt, c);
 }
 
 cudaError_t adamw_bulk_prepare(int* blocks_per_sm) {

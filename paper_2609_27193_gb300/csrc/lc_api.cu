@@ -975,6 +975,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     mp.nlayers = nlayers;
     mp.fault = ctx->d_fault;
     mp.stall_first = 0;
+    mp.static_tables = 1;
     MeasureParams& mpb = ctx->mpb;
     mpb = mp;
     mpb.cta_vec_begin = reinterpret_cast<const int64_t*>(base + o_ctav_b);

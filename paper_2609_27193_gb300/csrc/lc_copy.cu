@@ -432,6 +432,8 @@ __global__ void __launch_bounds__(kCopyThreads, 1) copy_bulk_kernel(CopyParams p
     __shared__ uint32_t s_abort;
     uint64_t x, xe;
     int first;
+    dependents_may_start();
+    dependency_wait();
     if (!cta_range(p, x, xe, first)) return;
     if (threadIdx.x == 0) {
         // an earlier CTA of this context gave up waiting: the copy's bytes
@@ -652,6 +654,8 @@ __global__ void __launch_bounds__(kCopyThreads, 1) copy_shift_kernel(CopyParams 
     __shared__ uint32_t s_abort;
     uint64_t x, xe;
     int first;
+    dependents_may_start();
+    dependency_wait();
     if (!cta_range(p, x, xe, first)) return;
     if (threadIdx.x == 0) {
         s_abort = p.fault_dev ? *reinterpret_cast<volatile const uint32_t*>(p.fault_dev) : 0u;
@@ -681,10 +685,7 @@ cudaError_t copy_occupancy(int* blocks_per_sm) {
 }
 
 cudaError_t launch_copy_bulk(const CopyParams& p, int grid, bool shifted, cudaStream_t s) {
-    cudaGetLastError();
-    if (shifted) copy_shift_kernel<<<grid, kCopyThreads, kBulkSmem, s>>>(p);
-    else copy_bulk_kernel<<<grid, kCopyThreads, kBulkSmem, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(shifted ? copy_shift_kernel : copy_bulk_kernel, grid, kCopyThreads, kBulkSmem, s, p);
 }
 
 cudaError_t copy_bulk_prepare(int* blocks_per_sm) {

@@ -608,7 +608,9 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
         for (int b = 0; b < kMBoxes; ++b) r.box.count[b] = 0u;
         mbar_init_fence();
     }
-    fin_prefetch(p, tables);
+    fin_prefetch(p, tables);   // before the wait: see static_tables
+    dependents_may_start();
+    dependency_wait();
     __syncthreads();
     if (threadIdx.x == 0) {
         measure_produce(p, ring, r);
@@ -644,10 +646,13 @@ cudaError_t launch_measure(const MeasureParams& p, int grid, bool write_ref, cud
 }
 
 cudaError_t launch_measure_bulk(const MeasureParams& p, int grid, bool write_ref, cudaStream_t s) {
-    cudaGetLastError();
-    if (write_ref) measure_bulk_kernel<true><<<grid, kMeasureThreads, kMeasureBulkSmem, s>>>(p);
-    else measure_bulk_kernel<false><<<grid, kMeasureThreads, kMeasureBulkSmem, s>>>(p);
-    return cudaGetLastError();
+    if (!p.static_tables) {   // the kernel before this one writes the tables: nothing could start early
+        cudaGetLastError();
+        measure_bulk_kernel<false><<<grid, kMeasureThreads, kMeasureBulkSmem, s>>>(p);
+        return cudaGetLastError();
+    }
+    return launch_dependent(write_ref ? measure_bulk_kernel<true> : measure_bulk_kernel<false>, grid, kMeasureThreads,
+                            kMeasureBulkSmem, s, p);
 }
 
 cudaError_t measure_bulk_prepare(int* blocks_per_sm) {

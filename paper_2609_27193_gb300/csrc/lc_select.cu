@@ -61,6 +61,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
     const int nsec_all = p.nsec;
     SectionDev sc;
     if (tid < nsec_all) sc = p.secs[tid];
+    dependents_may_start();
+    dependency_wait();
     const int64_t step = p.step_from_counter ? __ldcg(p.step_counter) + 1 : p.step;
     uint64_t run = 0, commit_work = 0, sec = 0, num = 0, den = 0;   // sec: sections | W sections << 32
     uint32_t cnt = 0, odd = 0;                                      // selected | nonfinite << 16; not exact in 2^53
@@ -232,9 +234,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
 }  // namespace
 
 cudaError_t launch_select(const SelectParams& p, cudaStream_t s) {
-    cudaGetLastError();
-    select_kernel<<<1, kSelectThreads, 0, s>>>(p);
-    return cudaGetLastError();
+    return launch_dependent(select_kernel, 1, kSelectThreads, 0, s, p);
 }
 
 }  // namespace lc
