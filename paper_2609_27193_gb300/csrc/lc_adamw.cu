@@ -567,10 +567,12 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             const OptSegDev od = opt[j.seg];
             for (int64_t q = j.k0 + tid; q < j.k1; q += kAConsumers) adam_scalar_vector(sd, od, q, c, dd, da);
         } else {
-            dd += double(ed);
-            da += double(ea);
-            ed = 0.f;
-            ea = 0.f;
+            if (__any_sync(0xffffffffu, ed != 0.f || ea != 0.f)) {   // zero where no chain kept them
+                dd += double(ed);
+                da += double(ea);
+                ed = 0.f;
+                ea = 0.f;
+            }
             run_flush<kAConsumerWarps>(r.box, st, warp, lane, dd, da, p.partials + j.slot);
             dd = 0.0;
             da = 0.0;

@@ -556,10 +556,12 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
             da += double(xa);
         }
         if (j.slot >= 0) {   // flush: this warp's share of the run
-            dd += double(ed);
-            da += double(ea);
-            ed = 0.f;
-            ea = 0.f;
+            if (__any_sync(0xffffffffu, ed != 0.f || ea != 0.f)) {   // zero where no chain kept them
+                dd += double(ed);
+                da += double(ea);
+                ed = 0.f;
+                ea = 0.f;
+            }
             run_flush<kMConsumerWarps - (WRITE_R ? 1 : 0)>(r.box, box, warp, lane, dd, da, p.partials + j.slot);
             box = box + 1 < kMBoxes ? box + 1 : 0;
             dd = 0.0;
