@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
         __syncthreads();
         uint64_t pb = run, pw = commit_work, ps = sec;
         cnt = 0;
-#pragma unroll
-        for (int w = 0; w < kSelWarps; ++w) {
+        const int warps = (p.nlayers - base + 31) / 32 < kSelWarps ? (p.nlayers - base + 31) / 32 : kSelWarps;
+        for (int w = 0; w < warps; ++w) {
             if (w < warp) {
                 pb += w_bytes[w];
                 pw += w_work[w];
