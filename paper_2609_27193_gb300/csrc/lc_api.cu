@@ -818,9 +818,9 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         std::vector<int32_t> cta_seg0, cta_slot0, layer_slot_begin;
         int32_t nslots = 0;
     };
-    auto partition = [&](int64_t grid, bool with_pool) {
+    auto partition = [&](int64_t grid, int64_t units_per_cta) {
         Partition pt;
-        pt.sh = partition_shape(V, grid, with_pool);
+        pt.sh = partition_shape(V, grid, units_per_cta);
         const size_t R = size_t(pt.sh.ranges());
         pt.cta_vec.resize(R + 1);
         pt.cta_seg0.resize(R);
@@ -832,10 +832,11 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     };
     int occ = 0;
     LC_CUDA(measure_occupancy(&occ));
-    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ), false);
+    const Partition pa = partition(int64_t(ctx->sms) * std::max(1, occ), 0);
     int bocc = 0;
     LC_CUDA(measure_bulk_prepare(&bocc));
-    const Partition pb = partition(int64_t(ctx->sms) * std::max(1, bocc) * LC_MEASURE_BULK_WAVES, true);
+    const Partition pb = partition(int64_t(ctx->sms) * std::max(1, bocc) * LC_MEASURE_BULK_WAVES,
+                                   LC_MEASURE_POOL_UNITS);
     const int64_t Rb = pb.sh.ranges(), G = pa.sh.G, Gb = pb.sh.G;
     ctx->measure_grid = int(G);
     ctx->measure_bulk_grid = int(Gb);

@@ -55,14 +55,15 @@ struct PartitionShape {
     int64_t ranges() const { return G + units; }
 };
 
-inline PartitionShape partition_shape(int64_t V, int64_t grid, bool with_pool) {
+// `units_per_cta`: at most so many pool units a CTA on average (0: no pool).
+inline PartitionShape partition_shape(int64_t V, int64_t grid, int64_t units_per_cta) {
     PartitionShape s;
     s.V = V;
     s.ngran = (V + LC_MEASURE_ALIGN_VECS - 1) / LC_MEASURE_ALIGN_VECS;
     s.G = s.ngran < grid ? s.ngran : grid;
     if (s.G < 1) s.G = 1;
-    if (with_pool) {
-        const int64_t pool = s.ngran * LC_MEASURE_POOL_PCT / 100, most = s.G * LC_MEASURE_POOL_UNITS;
+    if (units_per_cta > 0) {
+        const int64_t pool = s.ngran * LC_MEASURE_POOL_PCT / 100, most = s.G * units_per_cta;
         if (pool >= s.G * LC_MEASURE_POOL_MIN) {
             s.units = pool / LC_MEASURE_POOL_MIN < most ? pool / LC_MEASURE_POOL_MIN : most;
             s.pool = pool;
