@@ -1238,7 +1238,7 @@ extern "C" lc_status lc_last_select_info(const lc_ctx* ctx, lc_select_info* out)
     out->n_nonfinite = ctx->hdr.n_nonfinite;
     out->bytes = ctx->hdr.bytes;
     out->max_staleness = ctx->hdr.max_staleness;
-    out->weighted_staleness = ctx->hdr.weighted_staleness;
+    out->weighted_staleness = ctx->hdr.stale_den > 0.0 ? ctx->hdr.stale_num / ctx->hdr.stale_den : 0.0;
     return LC_OK;
 }
 

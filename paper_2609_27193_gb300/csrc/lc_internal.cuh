@@ -9,7 +9,7 @@ namespace lc {
 
 constexpr int kMeasureThreads = 256;   // threads per measure CTA
 constexpr int kCopyThreads = 256;      // threads per copy CTA
-constexpr int kSelectThreads = 512;    // the select kernel is a single CTA
+constexpr int kSelectThreads = 256;    // the select kernel is a single CTA
 
 // Work-range boundaries of the CTAs are rounded to these granules so that
 // every warp's 512-byte access starts on a 32-byte sector: a store that
@@ -151,7 +151,8 @@ struct ResultHeader {
     int32_t n_commit_desc;
     uint64_t commit_work;      // work-space bytes of the commit list
     int64_t max_staleness;
-    double weighted_staleness;
+    double stale_num;          // sum_l n_l (t - t_l) after the step, and sum_l n_l: their
+    double stale_den;          // quotient is taken on the host (a divide is slow here)
     uint32_t magic;
     uint32_t status;           // kStatusOk, or kStatusCapacity: nothing persisted
     uint64_t pack_bytes;       // bytes the pack moves: `bytes`, or 0 after kStatusCapacity

@@ -17,7 +17,7 @@ namespace lc {
 namespace {
 
 constexpr int kSelWarps = kSelectThreads / 32;
-constexpr double kExact = 9007199254740992.0;   // 2^53: whole numbers below it add exactly in binary64
+constexpr uint64_t kExact = uint64_t(1) << 53;   // whole numbers below it add exactly in binary64
 
 // Inclusive scan over the warp.
 __device__ __forceinline__ uint64_t warp_scan(uint64_t x, int lane) {
@@ -41,9 +41,14 @@ __device__ __forceinline__ uint64_t warp_add(uint64_t x) {
 // scan over the tile; and the decision goes straight to the pinned host block
 // that the host polls, header word last, instead of to a device block and a
 // copy and an event behind the kernel.  The decision over 6 M parameters in 6
-// layers takes 28 us of which this kernel is 7; with one thread laying out the
-// stream from shared memory and the copy it took 34.6 (146 layers: 33 and 46).
-__global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectParams p) {
+// layers takes 22.1 us, of which this kernel is about 4 once the sums are
+// there: 0.7 for the loads, 1.1 for Eq. 1's fp64 quotients (fp64 is slow here;
+// whole numbers and the host do the rest), 0.9 for the scans, 0.3 for the
+// lists and 0.7 for the host's block.  With one thread laying out the stream,
+// a copy and an event the decision took 6 us longer (146 layers: 13).  256
+// threads keep the CTA's registers at half an SM's, so that it finds room
+// beside other work.
+__global__ void __launch_bounds__(kSelectThreads, 2) select_kernel(const SelectParams p) {
     const ResultLayout L = result_layout(p.nlayers);
     uint8_t* const h_mask = p.host_block + L.mask_off;
     double* const h_u = reinterpret_cast<double*>(p.host_block + L.u_off);
@@ -59,8 +64,6 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
     __shared__ uint32_t w_cnt[kSelWarps], w_odd[kSelWarps];
 
     const int nsec_all = p.nsec;
-    SectionDev sc;
-    if (tid < nsec_all) sc = p.secs[tid];
     dependents_may_start();
     dependency_wait();
     const int64_t step = p.step_from_counter ? __ldcg(p.step_counter) + 1 : p.step;
@@ -98,7 +101,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
                 secs = uint64_t(uint32_t(s1 - s0)) | uint64_t(uint32_t(ws)) << 32;
             }
             // the staleness sums in whole numbers; past 2^53 they are taken again below
-            inexact = st < 0 || double(numel) * double(st) >= kExact || double(numel) >= kExact;
+            inexact = st < 0 || uint64_t(numel) >= kExact || __umul64hi(uint64_t(numel), uint64_t(st)) != 0 ||
+                      uint64_t(numel) * uint64_t(st) >= kExact;
             xn = inexact ? 0 : uint64_t(numel) * uint64_t(st);
             xd = inexact ? 0 : uint64_t(numel);
         }
@@ -143,7 +147,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
             cnt += w_cnt[w];
             odd |= w_odd[w];
         }
-        if (double(num) >= kExact || double(den) >= kExact) odd = 1;
+        if (num >= kExact || den >= kExact) odd = 1;
         nsel += int(cnt & 0xffffu);
         nnonfinite += int(cnt >> 16);
         if (in) {
@@ -183,7 +187,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
                 wd = __dadd_rn(wd, double(p.layer_numel[l]));
             }
         }
-        h.weighted_staleness = wd > 0.0 ? wn / wd : 0.0;
+        h.stale_num = wn;
+        h.stale_den = wd;
         h.magic = 0;
         h.status = fits ? kStatusOk : kStatusCapacity;
         h.pack_bytes = fits ? run : 0;
@@ -196,7 +201,7 @@ __global__ void __launch_bounds__(kSelectThreads) select_kernel(const SelectPara
         // go to its pack entries (and its W sections to its commit entries)
         const bool fused = p.fuse_commit != 0 && p.mode == 0;
         for (int j = tid; j < nsec_all; j += kSelectThreads) {
-            if (j != tid) sc = p.secs[j];
+            const SectionDev sc = p.secs[j];
             const LayerPlace q = place[sc.layer];
             if (!q.selected) continue;
             CopyDesc d;

@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("mode", ["snapshot", "accumulate"])
-@pytest.mark.parametrize("nlayers", [1, 31, 32, 33, 511, 512, 513, 1025])
+@pytest.mark.parametrize("nlayers", [1, 31, 32, 33, 255, 256, 257, 513, 1025])
 def test_layout_and_staleness_over_numbers_of_layers(nlayers, mode):
     """u injected per layer (D = u, A = 0, n = 1 with eps_w = 1): masks and
     statistics equal the oracle's, offsets the running block sizes, and the
