@@ -392,6 +392,7 @@ struct lc_ctx {
 
     // last decision
     bool have_select = false;
+    uint32_t select_calls = 0;
     ResultHeader hdr{};
     std::vector<uint8_t> mask;
     std::vector<uint64_t> offsets;
@@ -457,11 +458,11 @@ lc_status alloc_host_block(lc_ctx* ctx, uint8_t** host, uint8_t** dev) {
 // Polls the decision block's magic word, which the select kernel writes last,
 // until it is there or the configured timeout passes.  The stream is asked
 // now and then: an error on it would leave the word unwritten.
-lc_status wait_decision(lc_ctx* ctx, const uint32_t* magic, const char* what) {
+lc_status wait_decision(lc_ctx* ctx, const uint32_t* magic, uint32_t want, const char* what) {
     using clk = std::chrono::steady_clock;
     const auto t0 = clk::now();
     for (long spins = 1;; ++spins) {
-        if (__atomic_load_n(magic, __ATOMIC_ACQUIRE) == kResultMagic) return LC_OK;
+        if (__atomic_load_n(magic, __ATOMIC_ACQUIRE) == want) return LC_OK;
         if (spins % 256) continue;
         const auto ms = std::chrono::duration_cast<std::chrono::milliseconds>(clk::now() - t0).count();
         if (ms > ctx->cfg.timeout_ms)
@@ -472,7 +473,7 @@ lc_status wait_decision(lc_ctx* ctx, const uint32_t* magic, const char* what) {
             cudaGetLastError();
             return fail(LC_ERR_CUDA, "%s: %s", what, cudaGetErrorString(q));
         }
-        if (q == cudaSuccess && __atomic_load_n(magic, __ATOMIC_ACQUIRE) != kResultMagic)
+        if (q == cudaSuccess && __atomic_load_n(magic, __ATOMIC_ACQUIRE) != want)
             return fail(LC_ERR_CUDA, "%s: the decision was not written", what);
         if (ms > 20) std::this_thread::sleep_for(std::chrono::microseconds(50));
     }
@@ -1013,6 +1014,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     sp.commit_desc = reinterpret_cast<CopyDesc*>(base + o_cdesc);
     sp.nlayers = nlayers;
     sp.nsec = nsec;
+    sp.magic = kResultMagic;
     sp.mode = ctx->cfg.mode;
     sp.fuse_commit = ctx->cfg.fuse_commit;
     sp.eps_w = ctx->cfg.eps_w;
@@ -1197,18 +1199,20 @@ extern "C" lc_status lc_select(lc_ctx* ctx, double tau, int32_t max_staleness, u
     p.max_staleness = max_staleness;
     p.step = ctx->last_step;
     p.host_block = ctx->d_h_result;
-    uint32_t* magic = &reinterpret_cast<ResultHeader*>(ctx->h_result)->magic;
-    __atomic_store_n(magic, 0u, __ATOMIC_RELEASE);
+    // a number of its own: a call that ran out of time may have left a kernel
+    // behind that writes the block later
+    p.magic = kSelectMagic | (ctx->select_calls++ & (kSelectMagic - 1));
+    const uint32_t* magic = &reinterpret_cast<const ResultHeader*>(ctx->h_result)->magic;
     LC_CUDA(launch_select(p, ctx->stream));
     ctx->counters.kernel_launches += 1;
     ctx->counters.select_launches += 1;
     ctx->counters.d2h_bytes += ctx->rl.total;
-    LC_TRY(wait_decision(ctx, magic, "lc_select"));
+    LC_TRY(wait_decision(ctx, magic, p.magic, "lc_select"));
     LC_TRY(check_copy_fault(ctx, "lc_select"));
 
     ResultHeader h;
     std::memcpy(&h, ctx->h_result, sizeof h);
-    if (h.magic != kResultMagic || h.step != ctx->last_step || h.status != kStatusOk)
+    if (h.magic != p.magic || h.step != ctx->last_step || h.status != kStatusOk)
         return fail(LC_ERR_CUDA, "lc_select: decision block is corrupt");
     const uint8_t* m = ctx->h_result + ctx->rl.mask_off;
     const double* u = reinterpret_cast<const double*>(ctx->h_result + ctx->rl.u_off);

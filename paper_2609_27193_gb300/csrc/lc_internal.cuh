@@ -157,7 +157,8 @@ struct ResultHeader {
     uint32_t status;           // kStatusOk, or kStatusCapacity: nothing persisted
     uint64_t pack_bytes;       // bytes the pack moves: `bytes`, or 0 after kStatusCapacity
 };
-constexpr uint32_t kResultMagic = 0x4C43534Cu;
+constexpr uint32_t kResultMagic = 0x4C43534Cu;   // of a step read after its event
+constexpr uint32_t kSelectMagic = 0x80000000u;   // | number of the lc_select call that polls for it
 constexpr uint32_t kStatusOk = 0;
 constexpr uint32_t kStatusCapacity = 1;
 
@@ -211,6 +212,7 @@ struct SelectParams {
     int32_t max_staleness;
     int32_t nlayers;
     int32_t nsec;                    // sections of the layout
+    uint32_t magic;                  // written to the header last
     int32_t mode;                    // lc_drift_mode
     int32_t fuse_commit;
 };

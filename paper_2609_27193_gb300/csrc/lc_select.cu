@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kSelectThreads, 2) select_kernel(const SelectP
     __threadfence_system();   // this thread's part of the host block, before the header's magic word
     __syncthreads();
     if (tid == 0)
-        *reinterpret_cast<volatile uint32_t*>(&reinterpret_cast<ResultHeader*>(p.host_block)->magic) = kResultMagic;
+        *reinterpret_cast<volatile uint32_t*>(&reinterpret_cast<ResultHeader*>(p.host_block)->magic) = p.magic;
 }
 
 }  // namespace
