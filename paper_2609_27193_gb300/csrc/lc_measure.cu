@@ -258,10 +258,20 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 #endif
 constexpr int kMStages = LC_MEASURE_BULK_STAGES;
 constexpr uint32_t kMChunk = LC_MEASURE_BULK_CHUNK;      // bytes of W (and of R) per buffer
+// In accumulate mode a buffer that goes back to R by bulk store is filled less:
+// its next load waits for the store to have read it, and DRAM likes the loads
+// and stores in shorter turns.  1.2 G bf16 parameters in 146 layers: 1075 us
+// (6.9 TB/s; 1133 with full buffers of 24 KB, 1135 with 18, 1082 with 16, 1074
+// with 13 or 14, 1179 with 8), fp32 2128 (2205), 138 M 150.5 (156), 6 M 28.6
+// (29.0; 29.8 with 14 KB).
+#ifndef LC_MEASURE_ACC_CHUNK
+#define LC_MEASURE_ACC_CHUNK 15360
+#endif
 constexpr int kMConsumerWarps = kMeasureThreads / 32 - 1;   // warps 1.. consume (2.. in accumulate mode)
 constexpr uint32_t kMStage = 2 * kMChunk + 128;          // R's part has room for the window's extra vector
 constexpr size_t kMeasureBulkSmem = size_t(kMStages) * kMStage;
-static_assert(kMChunk % 16 == 0 && kMStages >= 2, "measure ring shape");
+static_assert(kMChunk % 16 == 0 && LC_MEASURE_ACC_CHUNK % 16 == 0 && LC_MEASURE_ACC_CHUNK <= kMChunk && kMStages >= 2,
+              "measure ring shape");
 
 // One job of a run: a chunk of n staged vectors (n may be 0), the elements at
 // the segment's edges (with the run's first job) and the flush (with its
@@ -292,6 +302,7 @@ struct MRing {
     RunBox<kMBoxes, kMConsumerWarps> box;
 };
 
+template <bool WRITE_R>
 __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r) {
     const uint32_t ring_s = smem_addr(ring);
     const uint32_t full_s = smem_addr(r.full), empty_s = smem_addr(r.empty);
@@ -338,12 +349,13 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
                 const int64_t q = (b << ve_log2) - sd.lead;
                 return q < sd.numel ? q : sd.numel;
             };
+            const int64_t most = (WRITE_R && sd.rshift == 0 ? LC_MEASURE_ACC_CHUNK : kMChunk) / 16;
             bool edges = true;
             do {
                 st = stage();
                 if (st < 0) break;
                 MJob& j = r.jobs[st];
-                const int64_t n = x < e ? (e - x < int64_t(kMChunk / 16) ? e - x : int64_t(kMChunk / 16)) : 0;
+                const int64_t n = x < e ? (e - x < most ? e - x : most) : 0;
                 j.na = j.nb = 0;
                 if (edges && lo < kf0) {
                     j.ea = first_elem(lo);
@@ -615,7 +627,7 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) measure_bulk_kernel(const 
     dependency_wait();
     __syncthreads();
     if (threadIdx.x == 0) {
-        measure_produce(p, ring, r);
+        measure_produce<WRITE_R>(p, ring, r);
     } else if (WRITE_R && threadIdx.x < 64) {
         if (threadIdx.x == 32) measure_store_r(p, ring, r);
     } else if (threadIdx.x >= 32) {
