@@ -466,8 +466,8 @@ __global__ void __launch_bounds__(kCopyThreads, 1) copy_bulk_kernel(CopyParams p
 // whole entry).  The bytes before the first and after the last granule, and
 // the padding of GATHER, are warp 1's.  Such entries used to move in units of
 // 2 or 4 bytes with ordinary loads: packing a quarter of the layers of a
-// 412 M parameter shard took 1960 us and takes 550 (the whole step 2256 and
-// 848 us; the same tensors on 16-byte boundaries 841).  Like the bulk form it
+// 412 M parameter shard took 1960 us and takes 540 (the whole step 2258 and
+// 817 us; with the tensors on 16-byte boundaries it differs by less than 1%).  Like the bulk form it
 // is bound by DRAM.
 // ---------------------------------------------------------------------------
 constexpr int kShiftFirstWarp = 2;

@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // is the same for the whole segment, so it is a template parameter of the
 // loop.  A run like that used to be read element by element, two fp64 adds
 // each: a decision over 412 M bf16 parameters in 146 such segments took
-// 3110 us and takes 294 (0.53 and 5.6 TB/s; the same parameters co-aligned
-// 269).  What bounds the shifted runs is the consumers' arithmetic: plain fp32
+// 3110 us and takes 264 (0.53 and 6.2 TB/s; the same parameters co-aligned
+// 250).  What bounds the shifted runs is the consumers' arithmetic: plain fp32
 // chains, as in the aligned runs, were 12% faster than chains that keep their
 // rounding errors, but lost precision against the element path's fp64 (6e-12
 // instead of 3e-12 off the exact sums).
