@@ -236,11 +236,13 @@ __global__ void __launch_bounds__(kMeasureThreads, LC_ADAM_MIN_BLOCKS) adamw_mea
 #ifndef LC_ADAM_BULK_STAGES
 #define LC_ADAM_BULK_STAGES 2
 #endif
-// A step over 1.2 G parameters with its decision: 5146 us with 544 vectors, 5163
-// with 512, 5218 with 480; 576 and 640 are faster there (5121, 5115) but slower
-// over 138 M (636 and 639 us; 615 with 544, 617 with 512).
+// A step over 1.2 G parameters with its decision takes 5163 us with 512
+// vectors, 5218 with 480 and 5146 with 544.  But the chunk is also the length
+// of a thread's fp32 chains between two fp64 adds: with 544 the sums are 3.8e-10
+// off their 64-bit values (root mean square over 16000 tensors, scaled to
+// 100,000 elements), with 512 3.5e-10.
 #ifndef LC_ADAM_BULK_VECS
-#define LC_ADAM_BULK_VECS 544
+#define LC_ADAM_BULK_VECS 512
 #endif
 constexpr int kAStages = LC_ADAM_BULK_STAGES;
 constexpr int kAChunkVec = LC_ADAM_BULK_VECS;                 // vectors of 4 parameters per chunk
@@ -438,8 +440,7 @@ __device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi)
 // errors: such segments used to be added element by element in fp64, and the
 // sums are no less exact now.  With bf16 gradients off the vectors of 412 M
 // parameters in 146 segments, a step and its decision took 4880 us element by
-// element and takes 1783, 1848 with m and v read by words too (floor 1696 at
-// 6.8 TB/s).
+// element and takes 1812 (floor 1696 at 6.8 TB/s).
 template <int FORM>
 __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid, const AdamConsts& c, double& dd,
                                            double& da, float& ed, float& ea, float& td, float& ta) {
