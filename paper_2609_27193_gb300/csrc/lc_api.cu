@@ -961,6 +961,9 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     LC_CUDA(cudaMalloc(&dev, total));
     ctx->d_tables = dev;
     LC_CUDA(cudaMemcpy(dev, host.data(), total, cudaMemcpyHostToDevice));
+    // A copy from pageable memory may return before its bytes have arrived, and the
+    // measure fetches tables from here before it waits for the kernel ahead of it.
+    LC_CUDA(cudaStreamSynchronize(nullptr));
     uint8_t* base = static_cast<uint8_t*>(dev);
 
     MeasureParams& mp = ctx->mp;
