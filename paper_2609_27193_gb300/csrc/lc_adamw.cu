@@ -437,8 +437,8 @@ __device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi)
 // up with w's vectors.  Otherwise the gradient (and in kALoose m and v) starts
 // where it likes: its staged words are read, and m's and v's written back, one
 // by one (four-way bank conflicts), and the Eq. 1 chains keep their rounding
-// errors: such segments used to be added element by element in fp64, and the
-// sums are no less exact now.  With bf16 gradients off the vectors of 412 M
+// errors (CompSum): such segments used to be added element by element in fp64,
+// and the sums are within the last place of fp64 of those.  With bf16 gradients off the vectors of 412 M
 // parameters in 146 segments, a step and its decision took 4880 us element by
 // element and takes 1812 (floor 1696 at 6.8 TB/s).
 template <int FORM>
@@ -453,7 +453,7 @@ __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid,
     uint8_t* Vb = buf + 2 * kAPart + ov;
     const uint8_t* G = buf + 3 * kAPart + og;
     float ad[4] = {0.f, 0.f, 0.f, 0.f}, aa[4] = {0.f, 0.f, 0.f, 0.f};
-    CompSums<2> cd, ca;
+    CompSum cd, ca;
     for (int q = tid; q < n; q += kAConsumers) {
         const uint4 pw = W[q];
         const uint4 mw = MOMENTS ? reinterpret_cast<const uint4*>(Mb)[q]
@@ -496,9 +496,9 @@ __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid,
             for (int e = 0; e < 4; ++e) big = fmaxf(big, fmaxf(fabsf(pn[e] - pv[e]), fabsf(pv[e])));
             const bool fine = big < 1e37f;
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                cd.add(e, fine ? fabsf(pn[e] - pv[e]) : 0.f);
-                ca.add(e, fine ? fabsf(pv[e]) : 0.f);
+            for (int e = 0; e < 4; e += 2) {
+                cd.add(F2::of(fine ? fabsf(pn[e] - pv[e]) : 0.f, fine ? fabsf(pn[e + 1] - pv[e + 1]) : 0.f));
+                ca.add(F2::of(fine ? fabsf(pv[e]) : 0.f, fine ? fabsf(pv[e + 1]) : 0.f));
             }
             if (!fine) {                    // near the end of fp32's range, or infinite
 #pragma unroll
@@ -530,12 +530,8 @@ __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid,
         td = (ad[0] + ad[1]) + (ad[2] + ad[3]);
         ta = (aa[0] + aa[1]) + (aa[2] + aa[3]);
     } else {
-        cd.reduce();
-        ca.reduce();
-        td = cd.s[0];
-        ta = ca.s[0];
-        ed += cd.e[0];
-        ea += ca.e[0];
+        cd.total(td, ed);
+        ca.total(ta, ea);
     }
 }
 
@@ -546,7 +542,6 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
     const int tid = int(threadIdx.x) - 32 * kAFirstConsumerWarp;
     const int warp = tid >> 5, lane = tid & 31;
     double dd = 0.0, da = 0.0;
-    float ed = 0.f, ea = 0.f;   // rounding errors of the run's compensated chains
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kAStages);
         const uint32_t parity = uint32_t((k / kAStages) & 1);
@@ -560,6 +555,7 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             break;
         }
         float td = 0.f, ta = 0.f;   // the chunk's sums
+        float ed = 0.f, ea = 0.f;   // with their rounding errors, where the chains keep them
         if (j.kind == kAJobChunk) {
             uint8_t* buf = ring + size_t(st) * kAStage;
             if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, ed, ea, td, ta);
@@ -572,20 +568,19 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             const OptSegDev od = opt[j.seg];
             for (int64_t q = j.k0 + tid; q < j.k1; q += kAConsumers) adam_scalar_vector(sd, od, q, c, dd, da);
         } else {
-            if (__any_sync(0xffffffffu, ed != 0.f || ea != 0.f)) {   // zero where no chain kept them
-                dd += double(ed);
-                da += double(ea);
-                ed = 0.f;
-                ea = 0.f;
-            }
             run_flush<kAConsumerWarps>(r.box, st, warp, lane, dd, da, p.partials + j.slot);
             dd = 0.0;
             da = 0.0;
         }
         mbar_arrive_warp(done_s + 8 * st, lane);
         after_handback(td, ta);
-        dd += double(td);
-        da += double(ta);
+        if (j.kind == kAJobChunk && j.form != kALined) {
+            dd += double(td) + double(ed);
+            da += double(ta) + double(ea);
+        } else {
+            dd += double(td);
+            da += double(ta);
+        }
     }
 }
 

@@ -796,7 +796,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
 
     // measure work space: 16-byte virtual vectors
     std::vector<SegDev> sd(nseg);
-    int64_t V = 0;
+    int64_t V = 0, shifted = 0;   // vectors; those of segments whose R is shifted
     for (int32_t i = 0; i < nseg; ++i) {
         const lc_segment& s = ctx->segs[i];
         const int esz_log2 = s.w_dtype == LC_BF16 ? 1 : 2;
@@ -812,6 +812,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
         d.nvec = (int64_t(d.lead) + s.numel + ve - 1) / ve;
         d.vec_begin = V;
         V += d.nvec;
+        if (d.rshift) shifted += d.nvec;
     }
     struct Partition {
         PartitionShape sh;
@@ -821,7 +822,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     };
     auto partition = [&](int64_t grid, int64_t units_per_cta) {
         Partition pt;
-        pt.sh = partition_shape(V, grid, units_per_cta);
+        pt.sh = partition_shape(V, grid, units_per_cta, shifted);
         const size_t R = size_t(pt.sh.ranges());
         pt.cta_vec.resize(R + 1);
         pt.cta_seg0.resize(R);

@@ -234,11 +234,16 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // is the same for the whole segment, so it is a template parameter of the
 // loop.  A run like that used to be read element by element, two fp64 adds
 // each: a decision over 412 M bf16 parameters in 146 such segments took
-// 3110 us and takes 264 (0.53 and 6.2 TB/s; the same parameters co-aligned
-// 250).  What bounds the shifted runs is the consumers' arithmetic: plain fp32
-// chains, as in the aligned runs, were 12% faster than chains that keep their
-// rounding errors, but lost precision against the element path's fp64 (6e-12
-// instead of 3e-12 off the exact sums).
+// 3110 us and takes 304 (0.53 and 5.4 TB/s; the same parameters co-aligned
+// 255).  What bounds the shifted bf16 runs is the consumers' arithmetic: plain
+// fp32 chains, as in the aligned runs, would be a sixth faster, but the sums
+// had fp64's precision before and plain chains lose it (6e-12 off the exact
+// sums instead of 3e-12 on ordinary weights, 7e-10 on magnitudes over 30
+// binades).  With chains that recovered an error only where the sum was the
+// larger operand a decision took 271 us; they were 4e-13 off on ordinary
+// weights and 7e-10 on the wide ones.  Their loops are short (unrolled twice, one
+// pair of chains): with four pairs 345 us, unrolled four times 406 (both with
+// the usual pool; as it is now 332), seven times 590.
 //
 // Warps 1..7 consume every job in order: each thread adds its 16-byte vectors
 // of the chunk into fp32 lanes (at most ceil(chunk vectors / 224) terms before
@@ -404,23 +409,18 @@ __device__ void measure_produce(const MeasureParams& p, uint8_t* ring, MRing& r)
 }
 
 template <int ESZ_LOG2>
-__device__ __forceinline__ void accumulate_comp(const uint4& w, const uint4& r, CompSums<ESZ_LOG2>& cd,
-                                                CompSums<ESZ_LOG2>& ca) {
+__device__ __forceinline__ void accumulate_comp(const uint4& w, const uint4& r, CompSum& cd, CompSum& ca) {
     const uint32_t wv[4] = {w.x, w.y, w.z, w.w};
     const uint32_t rv[4] = {r.x, r.y, r.z, r.w};
+    auto pair = [](const uint32_t (&x)[4], int j) {
+        return ESZ_LOG2 == 1 ? F2::of(bf16_lo(x[j]), bf16_hi(x[j]))
+                             : F2::of(__uint_as_float(x[2 * j]), __uint_as_float(x[2 * j + 1]));
+    };
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if constexpr (ESZ_LOG2 == 1) {
-            const float r0 = bf16_lo(rv[j]), r1 = bf16_hi(rv[j]);
-            cd.add(2 * j, fabsf(bf16_lo(wv[j]) - r0));
-            cd.add(2 * j + 1, fabsf(bf16_hi(wv[j]) - r1));
-            ca.add(2 * j, fabsf(r0));
-            ca.add(2 * j + 1, fabsf(r1));
-        } else {
-            const float r0 = __uint_as_float(rv[j]);
-            cd.add(j, fabsf(__uint_as_float(wv[j]) - r0));
-            ca.add(j, fabsf(r0));
-        }
+    for (int j = 0; j < (8 >> ESZ_LOG2); ++j) {
+        const F2 w2 = pair(wv, j), r2 = pair(rv, j);
+        cd.add((w2 - r2).abs());
+        ca.add(r2.abs());
     }
 }
 
@@ -446,12 +446,15 @@ __device__ __noinline__ double2 staged_elements(const uint8_t* W, const uint8_t*
 // first and last R vectors are only partly its own and are stored by
 // elements.  No other chunk reads or writes those elements of R.
 //
-// The fp32 chains keep their rounding errors (comp_add): these runs used to
-// be added element by element in fp64, and the sums are no less exact now.
+// The fp32 chains keep their rounding errors (CompSum): these runs used to be
+// added element by element in fp64.  Against the exact sums of the same fp32
+// terms, tensors of 100 to 1 M elements, both ways give bf16 sums without any
+// error for normally distributed weights, and up to 4e-16 for magnitudes
+// spread over 30 to 36 binades; fp32 sums 2e-16 and up to 6e-16 (4e-16 in fp64).
 template <int ESZ_LOG2, int SH, bool WRITE_R, int NT>
 __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int n, int tid, uint8_t* r_out,
                                             double& dd, double& da, float& ed, float& ea, float& td, float& ta) {
-    CompSums<ESZ_LOG2> cd, ca;
+    CompSum cd, ca;
 #pragma unroll 2
     for (int v = tid; v < n; v += NT) {
         const uint4 w = W[v];
@@ -477,15 +480,10 @@ __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int 
             }
         }
     }
-    cd.reduce();
-    ca.reduce();
-    td = ta = 0.f;
-    if (isfinite(cd.s[0]) && isfinite(ca.s[0])) {
-        td = cd.s[0];
-        ta = ca.s[0];
-        ed += cd.e[0];
-        ea += ca.e[0];
-    } else {
+    cd.total(td, ed);
+    ca.total(ta, ea);
+    if (!(isfinite(td) && isfinite(ta))) {
+        td = ta = ed = ea = 0.f;
         const double2 x = staged_elements<ESZ_LOG2>(reinterpret_cast<const uint8_t*>(W),
                                                     reinterpret_cast<const uint8_t*>(R) + SH, n, tid, NT);
         dd += x.x;
@@ -525,7 +523,6 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
     const int tid = int(threadIdx.x) - 32 * kFirstWarp;
     const int warp = tid >> 5, lane = tid & 31;
     double dd = 0.0, da = 0.0;
-    float ed = 0.f, ea = 0.f;   // rounding errors of the run's compensated chains
     int box = 0;                // of the next flush, the same in every warp
     for (uint64_t k = 0;; ++k) {
         const int st = int(k % kMStages);
@@ -539,6 +536,7 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
         float xd = 0.f, xa = 0.f;   // this thread's element of the segment's edges
         if (tid < j.na + j.nb) edge_element<WRITE_R>(p.segs[j.seg], tid < j.na ? j.ea + tid : j.eb + (tid - j.na), xd, xa);
         float td = 0.f, ta = 0.f;     // and its chunk's sums
+        float ed = 0.f, ea = 0.f;     // with their rounding errors, where the chains keep them
         if (j.n > 0) {
             const uint4* W = reinterpret_cast<const uint4*>(ring + size_t(st) * kMStage);
             const uint4* R = W + kMChunk / 16;
@@ -561,19 +559,18 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
         }
         mbar_arrive_warp(empty_s + 8 * st, lane);
         after_handback(td, ta);
-        dd += double(td);
-        da += double(ta);
+        if (j.rshift) {
+            dd += double(td) + double(ed);
+            da += double(ta) + double(ea);
+        } else {
+            dd += double(td);
+            da += double(ta);
+        }
         if (tid < j.na + j.nb) {
             dd += double(xd);
             da += double(xa);
         }
         if (j.slot >= 0) {   // flush: this warp's share of the run
-            if (__any_sync(0xffffffffu, ed != 0.f || ea != 0.f)) {   // zero where no chain kept them
-                dd += double(ed);
-                da += double(ea);
-                ed = 0.f;
-                ea = 0.f;
-            }
             run_flush<kMConsumerWarps - (WRITE_R ? 1 : 0)>(r.box, box, warp, lane, dd, da, p.partials + j.slot);
             box = box + 1 < kMBoxes ? box + 1 : 0;
             dd = 0.0;

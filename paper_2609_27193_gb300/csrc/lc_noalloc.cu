@@ -311,11 +311,13 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         d.nvec = (int64_t(d.lead) + s.numel + ve - 1) / ve;
     }
     int64_t V = 0;
+    int64_t shifted = 0;   // vectors of segments whose R is shifted
     for (int32_t i = 0; i < nseg; ++i) {
         sd[i].vec_begin = V;
         V += sd[i].nvec;
+        if (sd[i].rshift) shifted += sd[i].nvec;
     }
-    const PartitionShape sh = partition_shape(V, bulk ? ds.bulk_grid : ds.max_grid, bulk ? kPoolUnits : 0);
+    const PartitionShape sh = partition_shape(V, bulk ? ds.bulk_grid : ds.max_grid, bulk ? kPoolUnits : 0, shifted);
     const TableLayout L = table_layout(size_t(nseg), size_t(nlayers), size_t(sh.ranges()));
     if (sh.ranges() > kMaxRanges || L.bytes > kTableBytes)
         return err(LC_ERR_CUDA, "lc_measure_noalloc: internal table overflow");

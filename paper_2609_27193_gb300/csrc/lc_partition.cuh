@@ -31,6 +31,16 @@
 #ifndef LC_MEASURE_POOL_UNITS
 #define LC_MEASURE_POOL_UNITS 8
 #endif
+// Runs whose R is shifted cost the consumers more than aligned ones of the
+// same bytes, so equal shares take unequal times and the pool is larger where
+// they are a quarter of the vectors or more.  Decisions over 412 M parameters,
+// nearly all shifted: bf16 304 us (332 with the usual pool), accumulate mode
+// 413 (460), fp32 480 (481), accumulate mode 742 (811).  With fewer than 4
+// smallest units a CTA it shares worse than the usual pool (46 M parameters 57
+// instead of 55 us).
+#ifndef LC_MEASURE_POOL_PCT_SHIFTED
+#define LC_MEASURE_POOL_PCT_SHIFTED 30
+#endif
 
 namespace lc {
 
@@ -56,14 +66,17 @@ struct PartitionShape {
 };
 
 // `units_per_cta`: at most so many pool units a CTA on average (0: no pool).
-inline PartitionShape partition_shape(int64_t V, int64_t grid, int64_t units_per_cta) {
+// `shifted`: vectors of the segments whose R is shifted.
+inline PartitionShape partition_shape(int64_t V, int64_t grid, int64_t units_per_cta, int64_t shifted) {
     PartitionShape s;
     s.V = V;
     s.ngran = (V + LC_MEASURE_ALIGN_VECS - 1) / LC_MEASURE_ALIGN_VECS;
     s.G = s.ngran < grid ? s.ngran : grid;
     if (s.G < 1) s.G = 1;
     if (units_per_cta > 0) {
-        const int64_t pool = s.ngran * LC_MEASURE_POOL_PCT / 100, most = s.G * units_per_cta;
+        const int64_t more = s.ngran * LC_MEASURE_POOL_PCT_SHIFTED / 100, most = s.G * units_per_cta;
+        const int64_t pool = 4 * shifted >= V && more >= s.G * 4 * LC_MEASURE_POOL_MIN ? more
+                                                                              : s.ngran * LC_MEASURE_POOL_PCT / 100;
         if (pool >= s.G * LC_MEASURE_POOL_MIN) {
             s.units = pool / LC_MEASURE_POOL_MIN < most ? pool / LC_MEASURE_POOL_MIN : most;
             s.pool = pool;

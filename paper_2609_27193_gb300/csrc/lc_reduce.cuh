@@ -48,46 +48,59 @@ __device__ __forceinline__ void st_vec(void* p, uint4 v) {
 __device__ __forceinline__ float bf16_lo(uint32_t x) { return __uint_as_float(x << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t x) { return __uint_as_float(x & 0xffff0000u); }
 
-// a + b, its rounding error added to e (exact in any order of magnitude).
+// a + b, its rounding error added to e: Knuth's TwoSum, which recovers the
+// error exactly whichever operand is the larger.
 __device__ __forceinline__ float two_sum(float a, float b, float& e) {
     const float s = a + b, t = s - a;
     e += (a - (s - t)) + (b - t);
     return s;
 }
 
-// The same in three operations: exact once the sum a is at least as large as
-// the term b; before that within half the error that plain addition makes.
-__device__ __forceinline__ float fast_two_sum(float a, float b, float& e) {
-    const float s = a + b;
-    e += b - (s - a);
-    return s;
+// Two fp32 values in one 64-bit register pair; an operation on both is one
+// instruction.
+struct F2 {
+    uint64_t v;
+    static __device__ __forceinline__ F2 of(float lo, float hi) {
+        F2 r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+        return r;
+    }
+    __device__ __forceinline__ void split(float& lo, float& hi) const {
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+    }
+    __device__ __forceinline__ F2 abs() const { return F2{v & 0x7fffffff7fffffffull}; }
+};
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
 }
 
-// One chunk's fp32 chains of a thread with their rounding errors.  bf16
-// terms have 8 significant bits, so a chain rounds only where two terms are
-// more than 2^16 apart and the short form serves; fp32 terms round in every
-// addition and there are half as many of them per byte.
-template <int ESZ_LOG2>
-struct CompSums {
-    static constexpr int kLanes = 16 >> ESZ_LOG2;
-    float s[kLanes], e[kLanes];
-    __device__ __forceinline__ CompSums() {
-#pragma unroll
-        for (int i = 0; i < kLanes; ++i) { s[i] = 0.f; e[i] = 0.f; }
+// A chunk's sum of one thread: two fp32 chains and the rounding errors of
+// their additions, recovered exactly (two_sum) and added in fp32.  With
+// non-negative terms, n of them in a chain, the error words are below
+// n 2^-24 of the chain, so what they lose themselves is below n^2 2^-48 of it
+// (and nothing for bf16 values no more than 2^35 below the chain).  One pair of
+// chains: their latency is hidden by the other chain and warps, and the loops
+// that hold it stay short (lc_measure.cu has the times).
+struct CompSum {
+    F2 s{0}, e{0};
+    __device__ __forceinline__ void add(F2 x) {
+        const F2 n = s + x, t = n - s;
+        e = e + ((s - (n - t)) + (x - t));
+        s = n;
     }
-    __device__ __forceinline__ void add(int i, float x) {
-        s[i] = ESZ_LOG2 == 1 ? fast_two_sum(s[i], x, e[i]) : two_sum(s[i], x, e[i]);
-    }
-    // the chains' sum, left in s[0] and e[0]
-    __device__ __forceinline__ void reduce() {
-#pragma unroll
-        for (int k = kLanes / 2; k > 0; k >>= 1) {
-#pragma unroll
-            for (int i = 0; i < k; ++i) {
-                e[i] += e[i + k];
-                s[i] = two_sum(s[i], s[i + k], e[i]);
-            }
-        }
+    __device__ __forceinline__ void total(float& sum, float& err) const {
+        float a, b, c, d;
+        s.split(a, b);
+        e.split(c, d);
+        err = c + d;
+        sum = two_sum(a, b, err);
     }
 };
 
