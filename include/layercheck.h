@@ -237,6 +237,9 @@ lc_status lc_set_layer_sums_buffer(lc_ctx* ctx, double* sums_dev);
  * max_staleness: S_max >= 0 (0 persists every layer every step).
  * mask_out (nlayers bytes, 1 = persist), u_out (nlayers fp64), bytes_out:
  * host, each may be NULL.
+ * After TIMEOUT the step is still open and the call may be repeated, with
+ * the same tau and max_staleness or others: it decides as if it were the
+ * step's only one.
  * Errors: STATE (no lc_measure since the last select), INVALID_ARG,
  * TIMEOUT, CUDA. */
 lc_status lc_select(lc_ctx* ctx, double tau, int32_t max_staleness,

@@ -393,6 +393,7 @@ struct lc_ctx {
     // last decision
     bool have_select = false;
     uint32_t select_calls = 0;
+    bool select_launched = false;          // for the open step: a repeated lc_select starts from before it
     ResultHeader hdr{};
     std::vector<uint8_t> mask;
     std::vector<uint64_t> offsets;
@@ -924,6 +925,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     const size_t o_place = tp.take(sizeof(LayerPlace) * nlayers);
     const size_t o_accsave = tp.take(sizeof(double) * nlayers);
     const size_t o_tlsave = tp.take(sizeof(int64_t) * nlayers);
+    const size_t o_deltasave = tp.take(sizeof(double) * nlayers);
     const size_t o_stepctr = tp.take(sizeof(int64_t));
     ctx->rl = result_layout(nlayers);
     const size_t o_result = tp.take(sizeof(ResultHeader));
@@ -1010,6 +1012,7 @@ static lc_status register_layout_impl(lc_ctx* ctx, const lc_segment* segs, int32
     sp.layer_place = reinterpret_cast<LayerPlace*>(base + o_place);
     sp.acc_save = reinterpret_cast<double*>(base + o_accsave);
     sp.tl_save = reinterpret_cast<int64_t*>(base + o_tlsave);
+    sp.delta_save = reinterpret_cast<double*>(base + o_deltasave);
     sp.step_counter = reinterpret_cast<int64_t*>(base + o_stepctr);
     sp.capacity = UINT64_MAX;
     sp.step_from_counter = 0;
@@ -1063,6 +1066,7 @@ extern "C" lc_status lc_measure(lc_ctx* ctx, int64_t step) {
     LC_TRY(launch_measure_engine(ctx, ctx->stream));
     ctx->last_step = step;
     ctx->state = kMeasured;
+    ctx->select_launched = false;
     return LC_OK;
 }
 
@@ -1164,6 +1168,7 @@ extern "C" lc_status lc_adamw_step_measure(lc_ctx* ctx, int64_t step, const lc_a
     ctx->counters.measure_launches += 1;
     ctx->last_step = step;
     ctx->state = kMeasured;
+    ctx->select_launched = false;
     return LC_OK;
 }
 
@@ -1203,11 +1208,14 @@ extern "C" lc_status lc_select(lc_ctx* ctx, double tau, int32_t max_staleness, u
     p.max_staleness = max_staleness;
     p.step = ctx->last_step;
     p.host_block = ctx->d_h_result;
-    // a number of its own: a call that ran out of time may have left a kernel
-    // behind that writes the block later
+    // A call that ran out of time may have left a kernel behind, which still
+    // moves the step's state on and writes the block: the next one starts from
+    // the state before it, and its decision has a number of its own.
+    p.again = ctx->select_launched ? 1 : 0;
     p.magic = kSelectMagic | (ctx->select_calls++ & (kSelectMagic - 1));
     const uint32_t* magic = &reinterpret_cast<const ResultHeader*>(ctx->h_result)->magic;
     LC_CUDA(launch_select(p, ctx->stream));
+    ctx->select_launched = true;
     ctx->counters.kernel_launches += 1;
     ctx->counters.select_launches += 1;
     ctx->counters.d2h_bytes += ctx->rl.total;

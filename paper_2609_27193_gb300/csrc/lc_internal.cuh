@@ -203,6 +203,7 @@ struct SelectParams {
     CopyDesc* commit_desc;           // [nseg]
     double* acc_save;                // [nlayers] the step's accumulated drift (for a rollback)
     int64_t* tl_save;                // [nlayers] t_l before the step
+    double* delta_save;              // [nlayers] Delta_l before the step
     int64_t* step_counter;           // last step decided on the device
     double tau;
     double eps_w;
@@ -213,6 +214,8 @@ struct SelectParams {
     int32_t nlayers;
     int32_t nsec;                    // sections of the layout
     uint32_t magic;                  // written to the header last
+    int32_t again;                   // 1: a select of this step ran already and its decision was not read:
+                                     // decide from the state before it (tl_save, delta_save)
     int32_t mode;                    // lc_drift_mode
     int32_t fuse_commit;
 };

@@ -79,8 +79,8 @@ __global__ void __launch_bounds__(kSelectThreads, 2) select_kernel(const SelectP
         bool persist = false, nonfinite = false, inexact = false;
         if (in) {
             const double d = p.sums[3 * l], a = p.sums[3 * l + 1], n = p.sums[3 * l + 2];
-            const int64_t t_last = p.t_last[l], numel = p.layer_numel[l];
-            const double mult = p.tau_mult[l], before = p.mode == 1 ? p.delta[l] : 0.0;
+            const int64_t t_last = (p.again ? p.tl_save : p.t_last)[l], numel = p.layer_numel[l];
+            const double mult = p.tau_mult[l], before = p.mode == 1 ? (p.again ? p.delta_save : p.delta)[l] : 0.0;
             const uint64_t lb = p.layer_bytes[l], lw = p.layer_commit_work[l];
             const int32_t s0 = p.layer_sec_begin[l], s1 = p.layer_sec_begin[l + 1], ws = p.layer_wsec_count[l];
             const double u = (d / n) / (a / n + p.eps_w);                 // Eq. 1
@@ -90,8 +90,9 @@ __global__ void __launch_bounds__(kSelectThreads, 2) select_kernel(const SelectP
                       || step - t_last >= int64_t(p.max_staleness);       // §3.3
             p.acc_save[l] = acc;
             p.tl_save[l] = t_last;
+            p.delta_save[l] = before;
             p.delta[l] = persist ? 0.0 : acc;                             // Eq. 4
-            if (persist) p.t_last[l] = step;
+            if (persist || p.again) p.t_last[l] = persist ? step : t_last;
             h_mask[l] = persist ? 1 : 0;
             h_u[l] = u;
             st = persist ? 0 : step - t_last;
