@@ -361,7 +361,10 @@ typedef struct {
 /* Registers the gradient and model-copy pointers of every segment (§3.4.2:
  * the drift is computed on the optimizer update path).  Requires a layout
  * in LC_DRIFT_ACCUMULATE mode whose segments all have fp32 w and Adam
- * moments.  Errors: STATE (no layout, or snapshot mode), INVALID_ARG. */
+ * moments.  May be called again with other pointers: waits (bounded by
+ * timeout_ms) for the steps enqueued before, which use the old ones.
+ * Errors: STATE (no layout, or snapshot mode; again while the stream is
+ * being captured), INVALID_ARG, TIMEOUT, CUDA. */
 lc_status lc_register_optimizer(lc_ctx* ctx, const lc_optim_segment* segs, int32_t nseg);
 
 /* One AdamW step on every registered segment, in place on w, exp_avg and

@@ -1119,17 +1119,37 @@ extern "C" lc_status lc_register_optimizer(lc_ctx* ctx, const lc_optim_segment* 
         opt_device = opt_device && plain_device(o.grad) && (!o.model_copy || plain_device(o.model_copy));
     }
     // the bulk-load step: weights, moments, gradients and model copies all device memory
-    ctx->bulk_adam = ctx->cfg.copy_engine == LC_COPY_BULK && ctx->bulk_sources && opt_device;
-    if (ctx->bulk_adam) {
+    const bool bulk = ctx->cfg.copy_engine == LC_COPY_BULK && ctx->bulk_sources && opt_device;
+    if (bulk) {
         int occ = 0;
         LC_CUDA(adamw_bulk_prepare(&occ));
     }
-    if (!ctx->d_opt) {
-        void* p = nullptr;
-        LC_CUDA(cudaMalloc(&p, sizeof(OptSegDev) * ctx->nseg));
-        ctx->d_opt = static_cast<OptSegDev*>(p);
+    // Nothing orders the context's stream with the table's upload.  A step that
+    // was enqueued before still reads the present table, so it is waited for, and
+    // a copy from pageable memory may return before its bytes have arrived.
+    void* table = ctx->d_opt;
+    if (table) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        LC_CUDA(cudaStreamIsCapturing(ctx->stream, &capture));
+        if (capture != cudaStreamCaptureStatusNone)
+            return fail(LC_ERR_STATE, "lc_register_optimizer: the stream is being captured, its steps cannot be waited for");
+        cudaEvent_t ev;
+        LC_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        cudaError_t e = cudaEventRecord(ev, ctx->stream);
+        lc_status st = LC_OK;
+        if (e == cudaSuccess) st = wait_event(ev, ctx->cfg.timeout_ms, "lc_register_optimizer");
+        cudaEventDestroy(ev);
+        LC_CUDA(e);
+        LC_TRY(st);
+    } else {
+        LC_CUDA(cudaMalloc(&table, sizeof(OptSegDev) * ctx->nseg));
     }
-    LC_CUDA(cudaMemcpy(ctx->d_opt, od.data(), sizeof(OptSegDev) * ctx->nseg, cudaMemcpyHostToDevice));
+    cudaError_t e = cudaMemcpy(table, od.data(), sizeof(OptSegDev) * ctx->nseg, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    if (e != cudaSuccess && !ctx->d_opt) cudaFree(table);
+    LC_CUDA(e);
+    ctx->d_opt = static_cast<OptSegDev*>(table);
+    ctx->bulk_adam = bulk;
     return LC_OK;
 }
 
