@@ -613,10 +613,20 @@ lc_status lc_manifest_read(const char* dir, int32_t verify_blocks, lc_manifest_r
  * array: calls that overlap on the GPU (different streams, or different
  * host threads, without ordering between them) race and give wrong sums.
  *
+ * The waits of the bulk-load kernel (every W and R device memory) are
+ * bounded like those of lc_measure.  There is no context to report one that
+ * ran out: all 3*nlayers values are NaN then, the element counts among them,
+ * which no input can make NaN.
+ *
  * Errors: INVALID_ARG (layout, pointers), CAPACITY (nseg above
  * LC_NOALLOC_MAX_SEGMENTS or nlayers above LC_NOALLOC_MAX_LAYERS), CUDA. */
 lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_segment* segs,
                              int32_t nseg, int32_t nlayers, double* sums_out);
+
+/* lc_measure_noalloc with a test switch: debug_flags 0 or
+ * LC_DEBUG_MEASURE_STALL.  Errors: also INVALID_ARG (other flags). */
+lc_status lc_measure_noalloc_debug(int device, void* cuda_stream, const lc_segment* segs, int32_t nseg,
+                                   int32_t nlayers, double* sums_out, int32_t debug_flags);
 
 #ifdef __cplusplus
 }

@@ -130,6 +130,8 @@ SIGNATURES = {
     "lc_adamw_step_measure": (C.c_int, [ctx_p, C.c_int64, P(lc_adamw_hparams)]),
     "lc_measure_noalloc": (C.c_int, [C.c_int, C.c_void_p, P(lc_segment), C.c_int32, C.c_int32,
                                      C.c_void_p]),
+    "lc_measure_noalloc_debug": (C.c_int, [C.c_int, C.c_void_p, P(lc_segment), C.c_int32, C.c_int32,
+                                           C.c_void_p, C.c_int32]),
     "lc_copy_trace_enable": (C.c_int, [ctx_p, C.c_int32]),
     "lc_copy_trace_read": (C.c_int, [ctx_p, P(lc_copy_span), C.c_int64, P(C.c_int64), P(C.c_int64)]),
     "lc_crc32c": (C.c_uint32, [C.c_void_p, C.c_uint64, C.c_uint32]),

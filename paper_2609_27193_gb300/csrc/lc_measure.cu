@@ -658,6 +658,7 @@ cudaError_t launch_measure(const MeasureParams& p, int grid, bool write_ref, cud
 
 cudaError_t launch_measure_bulk(const MeasureParams& p, int grid, bool write_ref, cudaStream_t s) {
     if (!p.static_tables) {   // the kernel before this one writes the tables: nothing could start early
+        if (write_ref) return cudaErrorInvalidValue;   // no caller has such tables and an R to write
         cudaGetLastError();
         measure_bulk_kernel<false><<<grid, kMeasureThreads, kMeasureBulkSmem, s>>>(p);
         return cudaGetLastError();

@@ -230,10 +230,8 @@ bool is_device_memory(const void* p, int device, bool* plain, KnownMemory& known
     return true;
 }
 
-}  // namespace
-
-extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_segment* segs,
-                                        int32_t nseg, int32_t nlayers, double* sums_out) {
+lc_status measure_noalloc(int device, void* cuda_stream, const lc_segment* segs, int32_t nseg, int32_t nlayers,
+                          double* sums_out, bool stall) {
     set_last_error("");
     if (!segs || nseg <= 0) return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: no segments");
     if (nlayers <= 0) return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc: nlayers must be > 0");
@@ -362,6 +360,7 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
     p.units = int32_t(sh.units);
     p.fault = counters + 2;
     p.nan_on_fault = 1;
+    p.stall_first = stall ? 1 : 0;
     p.nseg = nseg;
     p.nlayers = nlayers;
     const cudaError_t e = bulk ? launch_measure_bulk(p, int(sh.G), false, stream)
@@ -371,4 +370,20 @@ extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_
         return err(LC_ERR_CUDA, "lc_measure_noalloc: launch failed: %s", cudaGetErrorString(e));
     }
     return LC_OK;
+}
+
+}  // namespace
+
+extern "C" lc_status lc_measure_noalloc(int device, void* cuda_stream, const lc_segment* segs,
+                                        int32_t nseg, int32_t nlayers, double* sums_out) {
+    return measure_noalloc(device, cuda_stream, segs, nseg, nlayers, sums_out, false);
+}
+
+extern "C" lc_status lc_measure_noalloc_debug(int device, void* cuda_stream, const lc_segment* segs, int32_t nseg,
+                                              int32_t nlayers, double* sums_out, int32_t debug_flags) {
+    if (debug_flags & ~LC_DEBUG_MEASURE_STALL) {
+        set_last_error("");
+        return err(LC_ERR_INVALID_ARG, "lc_measure_noalloc_debug: unknown debug flags %d", debug_flags);
+    }
+    return measure_noalloc(device, cuda_stream, segs, nseg, nlayers, sums_out, debug_flags != 0);
 }
