@@ -134,3 +134,78 @@ def test_large_layout_off_alignment():
     assert sums.cpu().numpy().reshape(2, 3).tolist() == want.tolist()
     assert lc.counters()["measure_pool_units"] > 0
     lc.close()
+
+
+EXTREMES = [("large", 2.0 ** 126), ("inf", float("inf")), ("nan", float("nan"))]
+
+
+@pytest.mark.parametrize("what,value", EXTREMES)
+@pytest.mark.parametrize("call", ["snapshot", "accumulate", "noalloc"])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_extreme_values_off_alignment(dtype, call, what, value):
+    """Weights, and references, near the end of fp32's range, infinite or NaN
+    in runs off one another's alignment, beside a run of ordinary ones: the
+    sums are what fp64 addition of the fp32 terms gives."""
+    torch = require_gpu()
+    import ctypes as C
+    import paper_2609_27193_gb300 as P
+    from paper_2609_27193_gb300 import _abi
+    n = 20000
+    tt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    pairs = [(_at(torch, n, tt, 4), _at(torch, n, tt, 12)) for _ in range(3)]
+    for x in (pairs[0][0], pairs[1][1]):
+        if what == "large":
+            x.fill_(value)
+        else:
+            x[n // 2] = value
+    pairs[2][0].fill_(0.5)
+    pairs[2][1].fill_(0.25)
+    segs = [P.segment(k, w, r) for k, (w, r) in enumerate(pairs)]
+    sums = torch.zeros(9, dtype=torch.float64, device="cuda")
+    if call == "noalloc":
+        _abi.check(P.library().lc_measure_noalloc(0, C.c_void_p(torch.cuda.current_stream().cuda_stream),
+                                                  (_abi.lc_segment * 3)(*segs), 3, 3, C.c_void_p(sums.data_ptr())))
+    else:
+        lc = P.LayerCheck(mode=P.LC_DRIFT_ACCUMULATE if call == "accumulate" else P.LC_DRIFT_SNAPSHOT)
+        lc.register_layout(segs, 3)
+        lc.set_layer_sums_buffer(sums)
+        lc.measure(1)
+    torch.cuda.synchronize()
+    x = n * value if what == "large" else value
+    want = [[x, 0.0, n], [x, x, n], [n * 0.25, n * 0.25, n]]
+    assert np.array_equal(sums.cpu().numpy().reshape(3, 3), want, equal_nan=True)
+    if call == "accumulate":
+        for w, r in pairs:
+            assert torch.equal(w.view(torch.uint8), r.view(torch.uint8))
+
+
+@pytest.mark.parametrize("what,value", EXTREMES)
+@pytest.mark.parametrize("form", ["gradients", "moments"])
+def test_fused_step_extreme_values_off_alignment(form, what, value):
+    """The same for the fused step's loose forms: no gradient, a decay that
+    halves every weight (an infinite one stays, so its update is NaN)."""
+    torch = require_gpu()
+    import paper_2609_27193_gb300 as P
+    n, at = 20000, 8 if form == "moments" else 0
+    segs, grads, ws = [], [], []
+    for k in range(2):
+        w, m, v, x = (_at(torch, n, torch.float32, o) for o in (0, at, at, 4))
+        if k == 1:
+            w.fill_(0.5)
+        elif what == "large":
+            w.fill_(value)
+        else:
+            w[n // 2] = value
+        segs.append(P.segment(k, w, None, m, v))
+        grads.append(x)
+        ws.append(w)
+    lc = P.LayerCheck(mode=P.LC_DRIFT_ACCUMULATE)
+    lc.register_layout(segs, 2)
+    lc.register_optimizer(grads)
+    sums = torch.zeros(6, dtype=torch.float64, device="cuda")
+    lc.set_layer_sums_buffer(sums)
+    lc.adamw_step_measure(1, lr=1.0, weight_decay=0.5)
+    torch.cuda.synchronize()
+    d, a = (n * value / 2, n * value) if what == "large" else (float("nan"), value)
+    assert np.array_equal(sums.cpu().numpy().reshape(2, 3), [[d, a, n], [n * 0.25, n * 0.5, n]], equal_nan=True)
+    assert (ws[1] == 0.25).all()
