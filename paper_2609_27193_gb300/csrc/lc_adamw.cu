@@ -443,7 +443,7 @@ __device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi)
 // element and takes 1812 (floor 1696 at 6.8 TB/s).
 template <int FORM>
 __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid, const AdamConsts& c, double& dd,
-                                           double& da, float& ed, float& ea, float& td, float& ta) {
+                                           double& da, float& td, float& ta) {
     constexpr bool LINED = FORM == kALined, MOMENTS = FORM != kALoose;
     const int n = j.n;
     uint4* W = reinterpret_cast<uint4*>(buf);
@@ -530,8 +530,11 @@ __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid,
         td = (ad[0] + ad[1]) + (ad[2] + ad[3]);
         ta = (aa[0] + aa[1]) + (aa[2] + aa[3]);
     } else {
+        float ed, ea;
         cd.total(td, ed);
         ca.total(ta, ea);
+        dd += double(ed);
+        da += double(ea);
     }
 }
 
@@ -555,12 +558,11 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
             break;
         }
         float td = 0.f, ta = 0.f;   // the chunk's sums
-        float ed = 0.f, ea = 0.f;   // with their rounding errors, where the chains keep them
         if (j.kind == kAJobChunk) {
             uint8_t* buf = ring + size_t(st) * kAStage;
-            if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, ed, ea, td, ta);
-            else if (j.form == kAMoments) adam_chunk<kAMoments>(j, buf, tid, c, dd, da, ed, ea, td, ta);
-            else adam_chunk<kALoose>(j, buf, tid, c, dd, da, ed, ea, td, ta);
+            if (j.form == kALined) adam_chunk<kALined>(j, buf, tid, c, dd, da, td, ta);
+            else if (j.form == kAMoments) adam_chunk<kAMoments>(j, buf, tid, c, dd, da, td, ta);
+            else adam_chunk<kALoose>(j, buf, tid, c, dd, da, td, ta);
             // the storer's bulk copies read what this thread wrote to the buffer
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         } else if (j.kind == kAJobScalar) {
@@ -574,13 +576,8 @@ __device__ void adam_consume(const MeasureParams& p, const OptSegDev* opt, const
         }
         mbar_arrive_warp(done_s + 8 * st, lane);
         after_handback(td, ta);
-        if (j.kind == kAJobChunk && j.form != kALined) {
-            dd += double(td) + double(ed);
-            da += double(ta) + double(ea);
-        } else {
-            dd += double(td);
-            da += double(ta);
-        }
+        dd += double(td);
+        da += double(ta);
     }
 }
 

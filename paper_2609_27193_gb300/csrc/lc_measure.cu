@@ -453,7 +453,7 @@ __device__ __noinline__ double2 staged_elements(const uint8_t* W, const uint8_t*
 // spread over 30 to 36 binades; fp32 sums 2e-16 and up to 6e-16 (4e-16 in fp64).
 template <int ESZ_LOG2, int SH, bool WRITE_R, int NT>
 __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int n, int tid, uint8_t* r_out,
-                                            double& dd, double& da, float& ed, float& ea, float& td, float& ta) {
+                                            double& dd, double& da, float& td, float& ta) {
     CompSum cd, ca;
 #pragma unroll 2
     for (int v = tid; v < n; v += NT) {
@@ -480,10 +480,14 @@ __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int 
             }
         }
     }
+    float ed, ea;
     cd.total(td, ed);
     ca.total(ta, ea);
-    if (!(isfinite(td) && isfinite(ta))) {
-        td = ta = ed = ea = 0.f;
+    if (isfinite(td) && isfinite(ta)) {
+        dd += double(ed);
+        da += double(ea);
+    } else {
+        td = ta = 0.f;
         const double2 x = staged_elements<ESZ_LOG2>(reinterpret_cast<const uint8_t*>(W),
                                                     reinterpret_cast<const uint8_t*>(R) + SH, n, tid, NT);
         dd += x.x;
@@ -493,23 +497,22 @@ __device__ __forceinline__ void shifted_run(const uint4* W, const uint4* R, int 
 
 template <bool WRITE_R, int NT>
 __device__ __forceinline__ void shifted_chunk(int esz_log2, int rshift, const uint4* W, const uint4* R, int n,
-                                              int tid, uint8_t* r_out, double& dd, double& da,
-                                              float& ed, float& ea, float& td, float& ta) {
+                                              int tid, uint8_t* r_out, double& dd, double& da, float& td, float& ta) {
     if (esz_log2 == 1) {
         switch (rshift) {
-            case 2: shifted_run<1, 2, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 4: shifted_run<1, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 6: shifted_run<1, 6, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 8: shifted_run<1, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 10: shifted_run<1, 10, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 12: shifted_run<1, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            default: shifted_run<1, 14, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 2: shifted_run<1, 2, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 4: shifted_run<1, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 6: shifted_run<1, 6, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 8: shifted_run<1, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 10: shifted_run<1, 10, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 12: shifted_run<1, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            default: shifted_run<1, 14, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
         }
     } else {
         switch (rshift) {
-            case 4: shifted_run<2, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            case 8: shifted_run<2, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
-            default: shifted_run<2, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, ed, ea, td, ta); break;
+            case 4: shifted_run<2, 4, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            case 8: shifted_run<2, 8, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
+            default: shifted_run<2, 12, WRITE_R, NT>(W, R, n, tid, r_out, dd, da, td, ta); break;
         }
     }
 }
@@ -536,12 +539,11 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
         float xd = 0.f, xa = 0.f;   // this thread's element of the segment's edges
         if (tid < j.na + j.nb) edge_element<WRITE_R>(p.segs[j.seg], tid < j.na ? j.ea + tid : j.eb + (tid - j.na), xd, xa);
         float td = 0.f, ta = 0.f;     // and its chunk's sums
-        float ed = 0.f, ea = 0.f;     // with their rounding errors, where the chains keep them
         if (j.n > 0) {
             const uint4* W = reinterpret_cast<const uint4*>(ring + size_t(st) * kMStage);
             const uint4* R = W + kMChunk / 16;
             if (j.rshift) {
-                shifted_chunk<WRITE_R, kThreads>(j.esz_log2, j.rshift, W, R, j.n, tid, j.r_out, dd, da, ed, ea, td, ta);
+                shifted_chunk<WRITE_R, kThreads>(j.esz_log2, j.rshift, W, R, j.n, tid, j.r_out, dd, da, td, ta);
             } else {
                 float ad[8], aa[8];
 #pragma unroll
@@ -559,13 +561,8 @@ __device__ void measure_consume(const MeasureParams& p, const uint8_t* ring, MRi
         }
         mbar_arrive_warp(empty_s + 8 * st, lane);
         after_handback(td, ta);
-        if (j.rshift) {
-            dd += double(td) + double(ed);
-            da += double(ta) + double(ea);
-        } else {
-            dd += double(td);
-            da += double(ta);
-        }
+        dd += double(td);
+        da += double(ta);
         if (tid < j.na + j.nb) {
             dd += double(xd);
             da += double(xa);
