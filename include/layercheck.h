@@ -168,7 +168,9 @@ typedef struct {
     int64_t measure_launches;
     int64_t select_launches;
     int64_t copy_launches;       /* pack / commit / restore copy kernels        */
-    uint64_t d2h_bytes;          /* bytes copied device -> host by the library  */
+    uint64_t d2h_bytes;          /* bytes that the library moved device -> host:
+                                    copies, and the decisions that the select
+                                    kernel stores to pinned memory              */
     uint64_t h2d_bytes;          /* bytes copied host -> device by the library  */
     int64_t bulk_copy_launches;  /* copy launches that ran on the bulk engine   */
     int64_t bulk_measure_launches; /* measure launches on the bulk engine       */

@@ -1315,9 +1315,11 @@ lc_status ensure_staging(lc_ctx* ctx) {
 
 // Bytes of a staged chunk of a `total`-byte pack: the first chunk's gather
 // overlaps no transfer, so a chunk is an eighth of the pack, down to 64 MB.
-// 530 MB in 14 layers of 138 M parameters: 2942 us in chunks of 33 MB or 66,
-// 3027 in slots of 256 MB (2746 at the link's 193 GB/s).  A restore's last
-// scatter is what its total leaves of a slot anyway: the same with both.
+// 530 MB in 14 layers of 138 M parameters: 2948-2955 us in chunks of 66 MB (33
+// the same), 3027-3030 in slots of 256 MB (2746 at the link's 193 GB/s), both
+// where the pinned pages take the whole rate; slow pages cost a run up to a
+// third more with either.  A restore's last scatter is what its total leaves of
+// a slot anyway: the same with both.
 uint64_t staged_chunk(const lc_ctx* ctx, uint64_t total) {
     return std::min(round_up(std::max<uint64_t>(total / 8, 64u << 20), 4096), ctx->slot_bytes);
 }

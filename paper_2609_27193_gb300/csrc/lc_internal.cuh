@@ -116,9 +116,10 @@ struct CopyParams {
 // `most` as long as each has LC_COPY_MIN_SHARE bytes.  A CTA costs a few
 // microseconds of latency whatever its share, so waves of small shares pay
 // them several times: the pack of 21 MB in a 6 M parameter step in eight waves
-// took 26 us of 70, in one wave of 69 KB shares the step takes 58.  Larger
-// packs are the same with 64 KB to 256 KB here (138 M parameters 299 us, 1.2 G
-// 2336-2342), smaller ones take longer with 32 KB.
+// took 26 us of 70, and one wave of 69 KB shares took 12 us off the step (50
+// now, with the other kernels as they are).  Larger packs are the same with
+// 64 KB to 256 KB here (138 M parameters 299 us, 1.2 G 2336-2342), smaller ones
+// take longer with 32 KB.
 #ifndef LC_COPY_MIN_SHARE
 #define LC_COPY_MIN_SHARE 131072
 #endif
@@ -270,9 +271,9 @@ cudaError_t copy_bulk_prepare(int* blocks_per_sm);
 // in the stream is still running (programmatic dependent launch): its CTAs take
 // the slots that the predecessor's leave, set up their barriers and fetch the
 // layout's constant tables, and wait (dependency_wait) for the predecessor to
-// be complete before they read or write anything else.  A decision over 6 M
-// parameters takes 26.2 instead of 28.5 us, a fused step 59 instead of 62, a
-// step over 138 M 291 instead of 296.
+// be complete before they read or write anything else.  That took a decision
+// over 6 M parameters from 28.5 to 26.2 us (22 now, with the kernels as they
+// are), a fused step from 62 to 59, a step over 138 M from 296 to 291.
 template <typename... P, typename... A>
 inline cudaError_t launch_dependent(void (*kernel)(P...), int grid, int threads, size_t smem, cudaStream_t s, A... args) {
     cudaLaunchAttribute attr{};

@@ -236,14 +236,14 @@ __global__ void __launch_bounds__(kMeasureThreads) measure_kernel(const MeasureP
 // each: a decision over 412 M bf16 parameters in 146 such segments took
 // 3110 us and takes 304 (0.53 and 5.4 TB/s; the same parameters co-aligned
 // 255).  What bounds the shifted bf16 runs is the consumers' arithmetic: plain
-// fp32 chains, as in the aligned runs, would be a sixth faster, but the sums
-// had fp64's precision before and plain chains lose it (6e-12 off the exact
-// sums instead of 3e-12 on ordinary weights, 7e-10 on magnitudes over 30
-// binades).  With chains that recovered an error only where the sum was the
-// larger operand a decision took 271 us; they were 4e-13 off on ordinary
-// weights and 7e-10 on the wide ones.  Their loops are short (unrolled twice, one
-// pair of chains): with four pairs 345 us, unrolled four times 406 (both with
-// the usual pool; as it is now 332), seven times 590.
+// fp32 chains, as in the aligned runs, would be a sixth faster, but these sums
+// had fp64's precision and plain chains lose it (6e-12 off the 64-bit sums of
+// ordinary weights instead of 3e-12).  With chains that recovered an error only
+// where the sum was the larger operand a decision took 271 us, and the sums
+// were 4e-13 off the exact ones of ordinary weights (now 0) and 7e-10 with
+// magnitudes over 30 binades (now 8e-17).  The loops are short, unrolled twice
+// over one pair of chains: with four pairs 345 us, unrolled four times 406 (both
+// with the usual pool of ranges, the present loop 332), seven times 590.
 //
 // Warps 1..7 consume every job in order: each thread adds its 16-byte vectors
 // of the chunk into fp32 lanes (at most ceil(chunk vectors / 224) terms before

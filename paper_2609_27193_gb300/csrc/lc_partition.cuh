@@ -47,9 +47,10 @@ namespace lc {
 // What a segment costs a CTA beside its bytes, in vectors: a job of its own
 // (and its edges), however small it is.  The CTAs' own ranges share the work
 // space by that measure, so that a range of several small tensors has fewer
-// bytes.  6 M parameters in 38 tensors: the decision takes 23.9 us (26.0 with
-// equal vectors, 25.2 with a cost of 768, 23.8 with 3072), with every tensor a
-// layer 26 (29.5); large models are the same.
+// bytes.  6 M parameters in 38 tensors: that took the decision from 26.0 us
+// (equal vectors) to 23.9 (25.2 with a cost of 768, 23.8 with 3072; 22 now, with
+// the select as it is), with every tensor a layer from 29.5 to 26; large models
+// are the same.
 #ifndef LC_MEASURE_SEG_COST
 #define LC_MEASURE_SEG_COST 1536
 #endif

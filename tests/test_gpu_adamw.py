@@ -141,7 +141,8 @@ def test_fused_adamw_bit_exact(layout, grad_dtype, engine):
     separate allocations (the 250,001- and 100,003-parameter segments span
     several chunks and end in a partial vector); "flat" starts tensors on
     odd offsets, so bf16 gradient vectors begin off 16 bytes and are peeled;
-    "skew" never lines up and goes element by element."""
+    "skew" never lines up: the bulk form reads such gradients at their own
+    offset, the thread form goes element by element."""
     _run(SIZES, layout, grad_dtype, engine=engine)
 
 

@@ -101,7 +101,7 @@ def test_measure_pool_of_ranges_with_odd_segments(alloc, mode):
     About 1.2 G elements in odd-sized segments of mixed dtypes over five
     layers, packed back to back (flat: most segments start off a 16-byte
     boundary, W and R alike) or with R shifted by one element (skew: W and R
-    never co-aligned, so every run goes element by element): enough for the
+    never co-aligned, so the consumers shift every run): enough for the
     library to use a pool, and the sums must match the oracle's.  In
     accumulate mode (six consumer warps and a storer that writes R <- W) R
     must equal W afterwards, bit for bit, in every tensor."""
