@@ -438,9 +438,9 @@ __device__ __forceinline__ void put_model(uint8_t* to, uint32_t lo, uint32_t hi)
 // where it likes: its staged words are read, and m's and v's written back, one
 // by one (four-way bank conflicts), and the Eq. 1 chains keep their rounding
 // errors (CompSum): such segments used to be added element by element in fp64,
-// and the sums are within the last place of fp64 of those.  With bf16 gradients off the vectors of 412 M
-// parameters in 146 segments, a step and its decision took 4880 us element by
-// element and takes 1812 (floor 1696 at 6.8 TB/s).
+// and the sums are within fp64's last place of those.  With bf16 gradients off
+// the vectors of 412 M parameters in 146 segments, a step and its decision took
+// 4880 us element by element and takes 1811 (floor 1696 at 6.8 TB/s).
 template <int FORM>
 __device__ __forceinline__ void adam_chunk(const AJob& j, uint8_t* buf, int tid, const AdamConsts& c, double& dd,
                                            double& da, float& td, float& ta) {
